@@ -92,9 +92,11 @@ typedef struct {
     int max_iters;     /* cap on total CG iterations of one solve (default 20000)                  */
     double inner_tol;  /* FP32 inner solve: relative residual reduction per refinement step
                           (default 1e-4; ignored by POISSON_FP64)                                  */
-    int tile;          /* FP32 inner-solve kernels.  0 = TMA plane-marching kernels, variant and
-                          z-chunk autotuned per shape (when nx % 8 == 0, else the column
-                          kernels); -1 = column kernels (plain loads); 10000000 F + 1000000 P +
+    int tile;          /* inner-solve kernels.  0 = Jacobi-PCG on chip when the grid fits the
+                          registers and shared memory of the GPU (about 1.2 million cells in
+                          FP32, half of that in FP64); else, FP32, the TMA plane-marching kernels,
+                          variant and z-chunk autotuned per shape (when nx % 8 == 0, else the
+                          column kernels); -1 = column kernels (plain loads); 10000000 F + 1000000 P +
                           100000 S + 10000 WS + 1000 CX + 100 CY + T = persistent marching
                           kernel with T rows of 32 threads, each owning CX x CY cells (tile
                           32 CX x CY T), a TMA producer warp when WS = 1 and an S-stage plane
@@ -199,10 +201,11 @@ int poisson_get_operator(poisson_t* h, double* bx, double* by, double* bz, doubl
 /* ------------------------------------------------------------------ batched solves
  * Many independent solves of uneven size driven together.  Every FP64 refinement step of the
  * batch is one batched residual kernel, one batched CG start and ONE cooperative persistent
- * PCG launch over all unfinished solves (captured in CUDA graphs, rebuilt when the batch
- * changes).  Solves submitted while a batch runs join it at its next refinement step
- * (continuous batching).  Handles with POISSON_FP64, POISSON_RBSSOR or nx % 8 != 0 are solved
- * one by one with poisson_solve when polled.
+ * PCG launch over all unfinished solves that stream their grids, and one over those held on
+ * chip (captured in CUDA graphs, rebuilt when the batch changes).  Solves submitted while a batch runs join it at its next refinement step
+ * (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or a grid that neither
+ * fits on chip nor has nx % 8 == 0 are solved with poisson_solve on worker threads;
+ * POISSON_RBSSOR and periodic handles that stream one by one when polled.
  * poisson_batch_submit enqueues n solves (handles[i] with its density already set, rhs[i],
  * p[i] in/out as in poisson_solve, tol[i]) and returns a ticket per solve.  The arrays must stay
  * valid, and the handles must not be used or destroyed, until poisson_poll reports the ticket.

@@ -5,15 +5,16 @@
 //   R: x64 += d for every job (k_batch_update), r32 = b - A64 x64 and its norms
 //      (k_batch_residual), scalars copied to the host;
 //   S: the inner-solve controls copied to the device, z = D^-1 r for every job
-//      (k_batch_init), ONE cooperative persistent PCG launch over all unfinished jobs
-//      (k_pcg on the batch's work list), scalars copied back.
+//      (k_batch_init), ONE cooperative persistent PCG launch over all unfinished jobs that
+//      stream their grids (k_pcg on the batch's work list) and one over those whose grids fit
+//      on chip (k_res, resident.cu), scalars copied back.
 // Between them the host decides, per job, whether it has converged (then its solution is copied
 // out and its ticket finishes) and sets the next inner tolerance.  Jobs submitted while a batch
 // runs join it at the next outer step (continuous batching): the job table, the work list and
 // the graphs are rebuilt then.  Finished jobs stay in the table, inactive, until the next
 // rebuild.  Jobs that cannot run in the batch's persistent kernel are solved with poisson_solve:
-// those whose solves launch only ordinary kernels (multigrid, FP64, column kernels) on worker
-// threads, several at once, each on its handle's own stream, so that small solves overlap on
+// those whose solves launch only ordinary kernels (multigrid, FP64, cut cells, column kernels;
+// on-chip handles among them take the column kernels there) on worker threads, several at once, each on its handle's own stream, so that small solves overlap on
 // the GPU; those that run a persistent cooperative launch of their own (periodic one-sweep,
 // red-black) one by one when polled -- two grid-filling cooperative launches in flight at once
 // could keep each other's CTAs from becoming resident, and their grid barriers would end by
@@ -32,6 +33,7 @@
 #include <vector>
 
 #include "alloc.h"
+#include "coop.h"
 #include "poisson.h"
 #include "capi_internal.h"
 #include "jobs.cuh"
@@ -79,10 +81,14 @@ struct Executor {
     Scalars* h_sc = nullptr;  // pinned
     double* d_part = nullptr;
     MarchCtl* h_ctl = nullptr;  // pinned
+    ResSolve* h_res = nullptr;  // pinned: the jobs that run on chip, in table order
+    std::vector<int> res_of;    // job -> its index in h_res, or -1
+    int nres = 0, nmarch = 0;
     int cap = 0;                // jobs the buffers hold
     size_t part_cap = 0;
     int blocks = 0;
     MarchPlan plan{};
+    ResPlan rplan{};
     cudaGraphExec_t gR = nullptr, gS = nullptr;
     bool dirty = true;
     // development trace (POISSON_TRACE): rebuilds and refinement steps, with their host time
@@ -112,6 +118,9 @@ struct Executor {
     void release() {
         release_graphs();
         march_plan_free(&plan);
+        res_plan_free(&rplan);
+        if (h_res) lib_free_host(h_res);
+        h_res = nullptr;
         if (d_jobs) lib_free(d_jobs);
         if (d_sc) lib_free(d_sc);
         if (d_part) lib_free(d_part);
@@ -229,6 +238,7 @@ struct Executor {
             J.b64 = H->b64; J.x64 = H->x64;
             J.d32 = H->d32; J.r32 = H->r32; J.z32 = H->z32; J.pa32 = H->p32a;
             J.sa32 = H->s32a; J.wa32 = H->w32a;
+            J.res = H->res ? 1 : 0;
             J.eta32 = H->eta32; J.eta16 = H->eta16;
             part += 2 * (size_t)J.blocks;
             J.tol2 = 0.25;
@@ -244,12 +254,17 @@ struct Executor {
             if (d_part) lib_free(d_part);
             if (h_jobs) lib_free_host(h_jobs);
             if (h_sc) lib_free_host(h_sc);
+            if (h_res) lib_free_host(h_res);
             d_jobs = nullptr; d_sc = nullptr; d_part = nullptr; h_jobs = nullptr; h_sc = nullptr;
+            h_res = nullptr;
+            cap = 0;
+            part_cap = 0;
             if (lib_malloc((void**)&d_jobs, sizeof(JobDev) * ncap) != cudaSuccess ||
                 lib_malloc((void**)&d_sc, sizeof(Scalars) * ncap) != cudaSuccess ||
                 lib_malloc((void**)&d_part, sizeof(double) * npart) != cudaSuccess ||
                 lib_malloc_host((void**)&h_jobs, sizeof(JobDev) * ncap) != cudaSuccess ||
-                lib_malloc_host((void**)&h_sc, sizeof(Scalars) * ncap) != cudaSuccess) {
+                lib_malloc_host((void**)&h_sc, sizeof(Scalars) * ncap) != cudaSuccess ||
+                lib_malloc_host((void**)&h_res, sizeof(ResSolve) * ncap) != cudaSuccess) {
                 cudaGetLastError();
                 return POISSON_ENOMEM;
             }
@@ -272,29 +287,47 @@ struct Executor {
             cudaMemcpyAsync(d_jobs, h_jobs, sizeof(JobDev) * nj, cudaMemcpyHostToDevice, st) !=
                 cudaSuccess)
             return POISSON_ECUDA;
-        // work list: every job of the table; variant: the one tuned for the largest job
-        std::vector<MarchSolve> ms(nj);
-        int big = 0;
+        // the jobs on chip, and the work list of the others (variant: the one tuned for the
+        // largest of them)
+        res_of.assign(nj, -1);
+        nres = nmarch = 0;
+        std::vector<MarchSolve> ms;
+        const poisson_t* HB = nullptr;
         for (int q = 0; q < nj; ++q) {
             poisson_t* H = table[q]->h;
-            ms[q] = MarchSolve{H->d, H->d32, H->r32, H->z32, H->p32a, H->p32b,
-                               bf16 ? (const void*)H->eta16 : (const void*)H->eta32, d_sc + q,
-                               H->s32a, H->s32b, H->w32a, H->w32b};
-            if (H->d.n > table[big]->h->d.n) big = q;
+            if (H->res) {
+                res_of[q] = nres;
+                ResSolve s = res_solve_of(H);
+                s.sc = d_sc + q;
+                h_res[nres++] = s;
+                continue;
+            }
+            ms.push_back(MarchSolve{H->d, H->d32, H->r32, H->z32, H->p32a, H->p32b,
+                                    bf16 ? (const void*)H->eta16 : (const void*)H->eta32, d_sc + q,
+                                    H->s32a, H->s32b, H->w32a, H->w32b});
+            ++nmarch;
+            if (!HB || H->d.n > HB->d.n) HB = H;
         }
-        const poisson_t* HB = table[big]->h;
-        const int var = HB->march ? HB->plan.variant : 0;
-        const int strat = HB->march ? HB->plan.strategy : MARCH_SPLIT_EQUAL;
-        int nsm = 0, dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const int nctas = std::max(1, march_occupancy(var, bf16)) * std::max(1, nsm);
-        int rc = march_plan_build(&plan, ms.data(), nj, var, bf16, nctas, strat, st);
-        // a lockstep deal can spread one CTA over too many solves: fall back to the equal split
-        if (rc == -1 && strat != MARCH_SPLIT_EQUAL)
-            rc = march_plan_build(&plan, ms.data(), nj, var, bf16, nctas, MARCH_SPLIT_EQUAL, st);
-        if (rc == -2) return POISSON_ENOMEM;
-        if (rc != 0) return POISSON_EINVAL;
+        if (nres) {
+            const int rc = res_plan_build(&rplan, h_res, nres, false, st);
+            if (rc == -2) return POISSON_ENOMEM;
+            if (rc != 0) return POISSON_EINVAL;
+        }
+        if (nmarch) {
+            const int var = HB->march ? HB->plan.variant : 0;
+            const int strat = HB->march ? HB->plan.strategy : MARCH_SPLIT_EQUAL;
+            int nsm = 0, dev = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+            const int nctas = std::max(1, march_occupancy(var, bf16)) * std::max(1, nsm);
+            int rc = march_plan_build(&plan, ms.data(), nmarch, var, bf16, nctas, strat, st);
+            // a lockstep deal can spread one CTA over too many solves: fall back to the equal split
+            if (rc == -1 && strat != MARCH_SPLIT_EQUAL)
+                rc = march_plan_build(&plan, ms.data(), nmarch, var, bf16, nctas,
+                                      MARCH_SPLIT_EQUAL, st);
+            if (rc == -2) return POISSON_ENOMEM;
+            if (rc != 0) return POISSON_EINVAL;
+        }
         return capture();
     }
 
@@ -307,9 +340,14 @@ struct Executor {
     }
     int seq_S() {
         cudaMemcpyAsync(d_jobs, h_jobs, sizeof(JobDev) * table.size(), cudaMemcpyHostToDevice, st);
-        launch_batch_init(d_jobs, (int)table.size(), blocks, st);
-        cudaMemcpyAsync(plan.ctl, h_ctl, sizeof(MarchCtl), cudaMemcpyHostToDevice, st);
-        const int rc = launch_march_pcg(plan, st);
+        int rc = 0;
+        if (nmarch) {
+            launch_batch_init(d_jobs, (int)table.size(), blocks, st);
+            cudaMemcpyAsync(plan.ctl, h_ctl, sizeof(MarchCtl), cudaMemcpyHostToDevice, st);
+            rc = launch_march_pcg(plan, st);
+        }
+        if (nres && rc == 0)
+            rc = launch_res(rplan, bf16 ? RES_ETA16 : RES_ETA32, h_res, nres, st);
         cudaMemcpyAsync(h_sc, d_sc, sizeof(Scalars) * table.size(), cudaMemcpyDeviceToHost, st);
         return rc;
     }
@@ -412,7 +450,16 @@ struct Executor {
             return POISSON_OK;
         }
         *h_ctl = MarchCtl{0u, nj, 0, 0, 0ull};
+        for (int q = 0; q < nj; ++q) {
+            if (res_of[q] < 0) continue;
+            ResSolve& s = h_res[res_of[q]];
+            s.active = h_jobs[q].active;
+            s.tol2 = h_jobs[q].tol2;
+            s.max_iter = h_jobs[q].max_iter;
+        }
+        if (nres && res_tags(&rplan, h_res, nres, st) != 0) return POISSON_ECUDA;
         if (gS) {
+            CoopOrder order(st);
             if (cudaGraphLaunch(gS, st) != cudaSuccess) return POISSON_ECUDA;
         } else if (seq_S() != 0) {
             return POISSON_ECUDA;
@@ -443,12 +490,13 @@ Executor* g_exec[2] = {nullptr, nullptr};  // FP32 and BF16 coefficients
 uint64_t g_next = 1;
 
 bool batchable(const poisson_t* H) {
-    // (periodic handles run their own padded one-sweep plans: solved one by one)
-    return H->opts.precision != POISSON_FP64 && H->opts.precond == POISSON_JACOBI &&
-           march_supported(H->d) && H->march && !H->periodic();
+    // (periodic handles that stream run their own padded one-sweep plans: solved one by one)
+    if (H->opts.precision == POISSON_FP64 || H->opts.precond != POISSON_JACOBI || H->cut()) return false;
+    return H->res || (march_supported(H->d) && H->march && !H->periodic());
 }
 
-// A handle whose solve launches no persistent cooperative kernel (see the header comment).
+// A handle whose solve launches no persistent cooperative kernel on a worker (see the header
+// comment).
 bool poolable(const poisson_t* H) { return !H->march && !H->rb; }
 
 // Worker threads for the pooled jobs, started with the first one.  Each takes a job, makes the
@@ -510,11 +558,15 @@ void worker() {
             cudaStreamWaitEvent(w, j->ready, 0);
             const cudaStream_t hs = j->h->st;
             j->h->st = w;
+            j->h->no_coop = true;
             rc = poisson_solve(j->h, j->rhs, j->p, j->tol, &st);
+            j->h->no_coop = false;
             j->h->st = hs;
         } else {
             cudaEventSynchronize(j->ready);
+            j->h->no_coop = true;
             rc = poisson_solve(j->h, j->rhs, j->p, j->tol, &st);
+            j->h->no_coop = false;
         }
         cudaEventDestroy(j->ready);
         std::lock_guard<std::mutex> lk(g_mu);  // poll reads the job under g_mu

@@ -10,6 +10,7 @@
 #include "internal.cuh"
 #include "march.h"
 #include "mg.h"
+#include "resident.h"
 
 struct poisson_s {
     pcg::Dims d{};
@@ -70,6 +71,12 @@ struct poisson_s {
     // the black Schur complement, compressed black vectors in the first and second halves of
     // z32 (x, p), p32a (u, both buffers), p32b (s^), s32a (w^); plan in `plan`
     bool rb = false;
+    // inner solves held on chip (resident.cu): Jacobi handles of grids that fit, tile option 0
+    bool res = false;
+    pcg::ResPlan rplan{};
+    pcg::ResSolve* res_host = nullptr;  // pinned staging of rplan.solves
+    // a worker thread solves the handle beside others: no launch that fills the GPU
+    bool no_coop = false;
     pcg::MarchPlan plan{};  // persistent work-list launch over this handle's grid
     pcg::MarchCtl* ctl_host = nullptr;  // pinned staging of plan.ctl
     // the column-kernel CG chunk (CG_CHUNK iterations of phases A and B) as a CUDA graph,
@@ -92,6 +99,8 @@ constexpr int PROF_PCG = PROF_RES + 2;         // event pair around a persistent
 constexpr int PROF_EVENTS = PROF_PCG + 2;
 
 cudaError_t& last_cuda_error();
+// The handle's solve as the on-chip launches see it (its controls and sums' place unset).
+pcg::ResSolve res_solve_of(const poisson_t* H);
 bool is_device_ptr(const void* p);
 // Whether a handle is in a batch job not yet reported by poisson_poll (batch.cu).
 bool batch_handle_busy(const poisson_t* H);

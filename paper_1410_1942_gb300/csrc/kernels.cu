@@ -858,6 +858,7 @@ __device__ __forceinline__ void batch_init_body(const JobDev& J, const Dims& d, 
 __global__ void __launch_bounds__(TX * TY) k_batch_init(const JobDev* jobs, int njobs) {
     __shared__ double smem[64];
     JOB_LOOP_BEGIN(J)
+    if (J.res) return;
     if (!J.active) {
         if (local_ == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
             J.sc->done = CONVERGED;

@@ -25,6 +25,7 @@
 #include "internal.cuh"
 #include "kernels.h"
 #include "march.h"
+#include "coop.h"
 #include "march_dev.cuh"
 #include "march_rb.h"
 #include "tma.cuh"
@@ -1358,9 +1359,8 @@ int launch_march_pcg(const MarchPlan& p, cudaStream_t st) {
     void* params[] = {&args};
     const void* k = p.periodic ? (p.bf16 ? v.k16p : v.k32p) : (p.bf16 ? v.k16 : v.k32);
     if (!k) return -1;
-    const cudaError_t e = cudaLaunchCooperativeKernel(k, dim3(p.nctas),
-                                                      dim3(32, v.tyt + v.ws), params,
-                                                      (size_t)(p.bf16 ? v.smem16 : v.smem32), st);
+    const cudaError_t e = coop_launch(k, dim3(p.nctas), dim3(32, v.tyt + v.ws), params,
+                                      (size_t)(p.bf16 ? v.smem16 : v.smem32), st);
     g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) {
         cudaGetLastError();
