@@ -95,8 +95,9 @@ typedef struct {
     int tile;          /* inner-solve kernels.  0 = Jacobi-PCG on chip when the grid fits the
                           registers and shared memory of the GPU (about 1.2 million cells in
                           FP32, half of that in FP64); else, FP32, the TMA plane-marching kernels,
-                          variant and z-chunk autotuned per shape (when nx % 8 == 0, else the
-                          column kernels); -1 = column kernels (plain loads); 10000000 F + 1000000 P +
+                          variant and z-chunk autotuned per shape (rows whose nx is not a multiple
+                          of 8 on the one-sweep ones, at a padded pitch; with periodic_x or red-black
+                          SSOR those rows take the column kernels); -1 = column kernels (plain loads); 10000000 F + 1000000 P +
                           100000 S + 10000 WS + 1000 CX + 100 CY + T = persistent marching
                           kernel with T rows of 32 threads, each owning CX x CY cells (tile
                           32 CX x CY T), a TMA producer warp when WS = 1 and an S-stage plane
@@ -203,8 +204,8 @@ int poisson_get_operator(poisson_t* h, double* bx, double* by, double* bz, doubl
  * batch is one batched residual kernel, one batched CG start and ONE cooperative persistent
  * PCG launch over all unfinished solves that stream their grids, and one over those held on
  * chip (captured in CUDA graphs, rebuilt when the batch changes).  Solves submitted while a batch runs join it at its next refinement step
- * (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or a grid that neither
- * fits on chip nor has nx % 8 == 0 are solved with poisson_solve on worker threads;
+ * (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or periodic x that
+ * neither fits on chip nor has nx % 8 == 0 are solved with poisson_solve on worker threads;
  * POISSON_RBSSOR and periodic handles that stream one by one when polled.
  * poisson_batch_submit enqueues n solves (handles[i] with its density already set, rhs[i],
  * p[i] in/out as in poisson_solve, tol[i]) and returns a ticket per solve.  The arrays must stay

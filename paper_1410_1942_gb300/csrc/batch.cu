@@ -168,8 +168,9 @@ struct Executor {
         if (copy_user(H->x64, j->p, bytes, dp ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                             st) != cudaSuccess)
             return POISSON_ECUDA;
-        if (cudaMemsetAsync(H->d32, 0, n * sizeof(float), st) != cudaSuccess ||
-            cudaMemsetAsync(H->p32a, 0, n * sizeof(float), st) != cudaSuccess)
+        const size_t inner = H->inner_cells() * sizeof(float);
+        if (cudaMemsetAsync(H->d32, 0, inner, st) != cudaSuccess ||
+            cudaMemsetAsync(H->p32a, 0, inner, st) != cudaSuccess)
             return POISSON_ECUDA;
         j->admitted = true;
         j->t0 = now_s();
@@ -238,6 +239,7 @@ struct Executor {
             J.b64 = H->b64; J.x64 = H->x64;
             J.d32 = H->d32; J.r32 = H->r32; J.z32 = H->z32; J.pa32 = H->p32a;
             J.sa32 = H->s32a; J.wa32 = H->w32a;
+            J.skip = H->pitch - H->d.nx;
             J.res = H->res ? 1 : 0;
             J.eta32 = H->eta32; J.eta16 = H->eta16;
             part += 2 * (size_t)J.blocks;
@@ -302,11 +304,13 @@ struct Executor {
                 h_res[nres++] = s;
                 continue;
             }
-            ms.push_back(MarchSolve{H->d, H->d32, H->r32, H->z32, H->p32a, H->p32b,
-                                    bf16 ? (const void*)H->eta16 : (const void*)H->eta32, d_sc + q,
-                                    H->s32a, H->s32b, H->w32a, H->w32b});
+            ms.push_back(march_solve_of(H));
+            ms.back().sc = d_sc + q;
             ++nmarch;
-            if (!HB || H->d.n > HB->d.n) HB = H;
+            // (rows of any length need a one-sweep variant: one of their handles gives it)
+            if (!HB || H->pitched() > HB->pitched() ||
+                (H->pitched() == HB->pitched() && H->d.n > HB->d.n))
+                HB = H;
         }
         if (nres) {
             const int rc = res_plan_build(&rplan, h_res, nres, false, st);

@@ -108,10 +108,13 @@ static void prof_add(poisson_t* H, int cls, cudaEvent_t a, cudaEvent_t b);
 // launch) with a persistent grid of (resident CTAs per SM) x (SMs) CTAs, its phases A and B
 // timed with events, and the fastest kept; the choice is cached per shape and coefficient type.
 // Shapes are tuned per size class: each dimension rounded up to a power of two (at least 16).
+// Handles that only the one-sweep kernels serve (periodic x, rows of any length) have choices of
+// their own.
 struct TuneKey {
-    int nx, ny, nz, bf16;
+    int nx, ny, nz, bf16, one_sweep;
     bool operator<(const TuneKey& o) const {
-        return std::tie(nx, ny, nz, bf16) < std::tie(o.nx, o.ny, o.nz, o.bf16);
+        return std::tie(nx, ny, nz, bf16, one_sweep) <
+               std::tie(o.nx, o.ny, o.nz, o.bf16, o.one_sweep);
     }
 };
 static int size_class(int v) {
@@ -120,7 +123,8 @@ static int size_class(int v) {
     return c;
 }
 static TuneKey tune_key(const Dims& d, bool bf16) {
-    return TuneKey{size_class(d.nx), size_class(d.ny), size_class(d.nz), bf16 ? 1 : 0};
+    return TuneKey{size_class(d.nx), size_class(d.ny), size_class(d.nz), bf16 ? 1 : 0,
+                   (d.walls & PERIODIC_X) || d.nx % 8 != 0};
 }
 static std::mutex g_tune_mu;
 static std::map<TuneKey, std::pair<int, int>> g_tuned;  // (variant, split strategy)
@@ -135,12 +139,16 @@ static int num_sms() {
     return n;
 }
 
-static MarchSolve march_solve_of(poisson_t* H) {
+MarchSolve march_solve_of(poisson_t* H) {
     const bool bf16 = H->opts.precision == POISSON_FP32_BF16COEF;
     if (H->periodic())  // the one-sweep kernels on padded rows (u: pu, s^: ps, w^: pw)
         return MarchSolve{H->d, H->d32, H->r32, H->pu[0], H->p32a, H->pu[1],
                           bf16 ? (const void*)H->peta16 : (const void*)H->peta32, H->sc,
                           H->ps[0], H->ps[1], H->pw[0], H->pw[1]};
+    if (H->pitched())
+        return MarchSolve{H->d, H->d32, H->r32, H->z32, H->p32a, H->p32b,
+                          bf16 ? (const void*)H->peta16 : (const void*)H->peta32, H->sc,
+                          H->s32a, H->s32b, H->w32a, H->w32b, H->pitch};
     return MarchSolve{H->d, H->d32, H->r32, H->z32, H->p32a, H->p32b,
                       bf16 ? (const void*)H->eta16 : (const void*)H->eta32, H->sc,
                       H->s32a, H->s32b, H->w32a, H->w32b};
@@ -159,8 +167,10 @@ static int build_plan(poisson_t* H, int var, int strategy) {
 static int march_run(poisson_t* H, bool bf16, double tol2, int max_iter, Scalars* result = nullptr) {
     cudaStream_t st = H->st;
     const Dims d = H->d;
-    cudaMemsetAsync(H->d32, 0, sizeof(float) * (size_t)d.n, st);
-    cudaMemsetAsync(H->p32a, 0, sizeof(float) * (size_t)d.n, st);
+    const size_t inner = sizeof(float) * H->inner_cells();
+    const int zskip = H->pitch - d.nx;
+    cudaMemsetAsync(H->d32, 0, inner, st);
+    cudaMemsetAsync(H->p32a, 0, inner, st);
     if (march_variant(H->plan.variant).family == 1) {
         // the start-up sweep reads s^ and w^ (times alpha = beta = 0): they must be finite
         if (H->periodic()) {
@@ -168,17 +178,17 @@ static int march_run(poisson_t* H, bool bf16, double tol2, int max_iter, Scalars
             cudaMemsetAsync(H->ps[0], 0, sizeof(float) * np, st);
             cudaMemsetAsync(H->pw[0], 0, sizeof(float) * np, st);
         } else {
-            cudaMemsetAsync(H->s32a, 0, sizeof(float) * (size_t)d.n, st);
-            cudaMemsetAsync(H->w32a, 0, sizeof(float) * (size_t)d.n, st);
+            cudaMemsetAsync(H->s32a, 0, inner, st);
+            cudaMemsetAsync(H->w32a, 0, inner, st);
         }
     }
     if (bf16)
         launch_cg_init<float, CoefEta<__nv_bfloat16>>(d, H->kc, CoefEta<__nv_bfloat16>{H->eta16},
                                                       H->r32, H->z32, H->sc, H->partials, tol2, 0,
-                                                      max_iter, st);
+                                                      max_iter, st, zskip);
     else
         launch_cg_init<float, CoefEta<float>>(d, H->kc, CoefEta<float>{H->eta32}, H->r32, H->z32,
-                                              H->sc, H->partials, tol2, 0, max_iter, st);
+                                              H->sc, H->partials, tol2, 0, max_iter, st, zskip);
     if (H->periodic()) launch_pad_rows_f32(d, PAD_V, H->z32, H->pu[0], st);  // u = D^-1 r, padded
     *H->ctl_host = MarchCtl{0u, 1, 0, 0, 0ull};
     CK(cudaMemcpyAsync(H->plan.ctl, H->ctl_host, sizeof(MarchCtl), cudaMemcpyHostToDevice, st));
@@ -200,8 +210,9 @@ static int setup_march(poisson_t* H) {
     if (forced > 0) {
         var = march_variant_of_tile(forced);
         strategy = march_split_of_tile(forced);
-        // periodic x runs on the one-sweep kernels only (others: the column kernels)
-        if (H->periodic() && march_variant(var).family != 1) return POISSON_OK;
+        // periodic x and rows of any length run on the one-sweep kernels only (others: the column
+        // kernels)
+        if ((H->periodic() || H->pitched()) && march_variant(var).family != 1) return POISSON_OK;
     } else {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(tune_key(d, bf16));
@@ -217,6 +228,10 @@ static int setup_march(poisson_t* H) {
         cudaStream_t st = H->st;
         if (bf16) launch_fill_bf16(n, H->eta16, 0.5f, st);
         else launch_fill_f32(n, H->eta32, 0.5f, st);
+        if (H->pitched()) {
+            if (H->peta32) launch_pitch_rows(d, H->pitch, H->eta32, H->peta32, st);
+            if (H->peta16) launch_pitch_rows(d, H->pitch, H->eta16, H->peta16, st);
+        }
         if (H->periodic()) {  // the one-sweep kernels read rho/2 from padded rows
             if (H->peta32) launch_pad_rows_f32(d, 4, H->eta32, H->peta32, st);
             if (H->peta16) launch_pad_rows_bf16(d, 8, H->eta16, H->peta16, st);
@@ -232,7 +247,8 @@ static int setup_march(poisson_t* H) {
         for (int cand = 0; cand < march_variant_count(); ++cand) {
             const MarchVariant mv = march_variant(cand);
             if (mv.cx != 2 || mv.family >= 2 || march_occupancy(cand, bf16) <= 0) continue;
-            if (H->periodic() && mv.family != 1) continue;  // only the one-sweep kernels wrap
+            // only the one-sweep kernels wrap, or take rows of any length
+            if ((H->periodic() || H->pitched()) && mv.family != 1) continue;
             for (int strat = 0; strat < MARCH_SPLITS; ++strat) {
                 if (build_plan(H, cand, strat) != 0) continue;
                 float t[2];
@@ -550,6 +566,14 @@ static bool res_wanted(const Dims& d, const poisson_opts& o) {
            res_supported(d, o.precision == POISSON_FP64);
 }
 
+// Columns per stored row of the inner vectors (poisson_s::pitch).
+static int pitch_wanted(const Dims& d, const poisson_opts& o, bool res) {
+    return o.precision != POISSON_FP64 && o.precond == POISSON_JACOBI && o.tile != -1 && !res &&
+                   march_supported(d)
+               ? row_pitch(d.nx)
+               : d.nx;
+}
+
 // Reduction partial slots of one column-kernel launch of the handle's grid.
 static size_t column_blocks(const Dims& d, int kc) {
     const dim3 g((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY, (d.nz + kc - 1) / kc);
@@ -579,6 +603,10 @@ static void for_each_array(poisson_t* H, F&& f) {
         else
             f((void**)&H->peta16, (size_t)(d.nx + 16) * d.ny * d.nz, sizeof(__nv_bfloat16));
     }
+    if (H->pitched()) {
+        if (o.precision == POISSON_FP32) f((void**)&H->peta32, H->inner_cells(), F4);
+        else f((void**)&H->peta16, H->inner_cells(), sizeof(__nv_bfloat16));
+    }
     if (o.dirichlet_walls) f((void**)&H->rinv2, N, D8);  // (not needed for periodic x)
     f((void**)&H->eta32, N, F4); f((void**)&H->eta16, N, sizeof(__nv_bfloat16));
     f((void**)&H->x64, N, D8); f((void**)&H->b64, N, D8);
@@ -587,9 +615,10 @@ static void for_each_array(poisson_t* H, F&& f) {
         f((void**)&H->r64, N, D8); f((void**)&H->z64, N, D8); f((void**)&H->p64a, N, D8);
         f((void**)&H->p64b, N, D8);
     } else {
-        for (float** q : {&H->d32, &H->r32, &H->z32, &H->p32a, &H->p32b}) f((void**)q, N, F4);
+        const size_t NP = H->inner_cells();
+        for (float** q : {&H->d32, &H->r32, &H->z32, &H->p32a, &H->p32b}) f((void**)q, NP, F4);
         if (!H->res)  // on chip: s^ and w^ never leave it
-            for (float** q : {&H->s32a, &H->s32b, &H->w32a, &H->w32b}) f((void**)q, N, F4);
+            for (float** q : {&H->s32a, &H->s32b, &H->w32a, &H->w32b}) f((void**)q, NP, F4);
     }
     f((void**)&H->sc, 1, sizeof(Scalars));
     f((void**)&H->partials, std::max<size_t>(2 * H->nblocks + 64, 4096), D8);
@@ -632,6 +661,7 @@ extern "C" int poisson_create(int nx, int ny, int nz, double h, const poisson_op
     cudaGetDevice(&H->device);
     H->nblocks = column_blocks(H->d, H->kc);
     H->res = res_wanted(H->d, o);
+    H->pitch = pitch_wanted(H->d, o, H->res);
 
     int rc = POISSON_OK;
     auto A = [&](int r) { if (rc == POISSON_OK) rc = r; };
@@ -670,7 +700,7 @@ extern "C" int poisson_create(int nx, int ny, int nz, double h, const poisson_op
         o.tile != -1 && !H->res && march_supported(H->d))
         A(setup_march(H));
     if (rc == POISSON_OK && o.precision != POISSON_FP64 && o.precond == POISSON_RBSSOR &&
-        o.omega == 1.0 && o.tile != -1 && march_supported(H->d) && !o.periodic_x)
+        o.omega == 1.0 && o.tile != -1 && march_supported(H->d) && nx % 8 == 0 && !o.periodic_x)
         A(setup_rb(H));
     if (rc != POISSON_OK) {
         free_state(H);
@@ -703,6 +733,7 @@ extern "C" int poisson_required_bytes(int nx, int ny, int nz, const poisson_opts
     probe.opts = o;
     probe.nblocks = column_blocks(dims, choose_kc(dims));
     probe.res = res_wanted(dims, o);
+    probe.pitch = pitch_wanted(dims, o, probe.res);
     size_t b = 0;
     for_each_array(&probe, [&](void**, size_t count, size_t es) { b += count * es; });
     if (o.precond == POISSON_MG) {
@@ -763,6 +794,10 @@ extern "C" int poisson_set_density(poisson_t* H, const double* F, double rho_air
     CK(cudaMemcpyAsync(&bad_host, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, H->st));
     CK(cudaStreamSynchronize(H->st));
     if (bad_host) return POISSON_EINVAL;  // left not ready: solves give ENOTREADY
+    if (H->pitched()) {
+        if (H->peta32) launch_pitch_rows(H->d, H->pitch, H->eta32, H->peta32, H->st);
+        if (H->peta16) launch_pitch_rows(H->d, H->pitch, H->eta16, H->peta16, H->st);
+    }
     if (H->periodic() && H->pu[0]) {
         // rho/2 in rows padded by its halo width (4 FP32 / 8 BF16 columns, 16 bytes)
         if (H->peta32) launch_pad_rows_f32(H->d, 4, H->eta32, H->peta32, H->st);
@@ -1103,7 +1138,7 @@ static int solve_mixed(poisson_t* H, const C32& c32, bool bf16, double tol, int*
         NvtxRange inner_range("inner solve");
         Scalars res;
         rc = POISSON_ECUDA;
-        bool inner_done = false, rb_used = false;
+        bool inner_done = false, rb_used = false, rows = false;
         if (H->res && !H->no_coop) {
             rc = res_run(H, target * target, H->opts.max_iters - total, &res);
             if (rc == POISSON_ECUDA) H->res = false;  // launch refused: use the column kernels
@@ -1123,6 +1158,7 @@ static int solve_mixed(poisson_t* H, const C32& c32, bool bf16, double tol, int*
             rc = march_run(H, bf16, target * target, H->opts.max_iters - total, &res);
             if (rc == POISSON_ECUDA) H->march = false;  // launch refused: use the column kernels
             else inner_done = true;
+            rows = inner_done && H->pitched();
         }
         if (!inner_done)
             rc = cg_loop_columns<float, C32>(H, c32, H->d32, H->r32, H->z32, H->p32a,
@@ -1132,7 +1168,8 @@ static int solve_mixed(poisson_t* H, const C32& c32, bool bf16, double tol, int*
         total += res.iter;
         // (the red-black solve's correction holds its red relaxation even after 0 iterations)
         if (res.iter > 0 || (rb_used && inner_done && res.done != BREAKDOWN && res.done != TIMEDOUT))
-            launch_update64(H->d.n, H->x64, H->d32, H->st);
+            rows ? launch_update64_rows(H->d, H->pitch, H->x64, H->d32, H->st)
+                 : launch_update64(H->d.n, H->x64, H->d32, H->st);
         CK(cudaGetLastError());
         if (res.done == TIMEDOUT) { status = POISSON_ETIMEOUT; break; }
         if (res.done == BREAKDOWN && res.iter == 0) { status = POISSON_EBREAKDOWN; break; }

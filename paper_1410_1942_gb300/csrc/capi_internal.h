@@ -41,6 +41,12 @@ struct poisson_s {
     float *pu[2] = {nullptr, nullptr}, *ps[2] = {nullptr, nullptr}, *pw[2] = {nullptr, nullptr};
     float* peta32 = nullptr;
     __nv_bfloat16* peta16 = nullptr;
+    // rows of any length on the one-sweep marching kernels (nx not a multiple of 8): the inner vectors
+    // but r32 and rho/2 (in peta32 / peta16) at this many columns per row while `march` is set; nx
+    // otherwise
+    int pitch = 0;
+    bool pitched() const { return pitch != d.nx; }
+    size_t inner_cells() const { return (size_t)pitch * d.ny * d.nz; }
     bool periodic() const { return (d.walls & pcg::PERIODIC_X) != 0; }
     bool cut() const { return vol64 != nullptr; }
     // rho / 2 per cell for the reduced-precision inner operator
@@ -101,6 +107,8 @@ constexpr int PROF_EVENTS = PROF_PCG + 2;
 cudaError_t& last_cuda_error();
 // The handle's solve as the on-chip launches see it (its controls and sums' place unset).
 pcg::ResSolve res_solve_of(const poisson_t* H);
+// The handle's arrays as the marching kernels see them.
+pcg::MarchSolve march_solve_of(poisson_t* H);
 bool is_device_ptr(const void* p);
 // Whether a handle is in a batch job not yet reported by poisson_poll (batch.cu).
 bool batch_handle_busy(const poisson_t* H);

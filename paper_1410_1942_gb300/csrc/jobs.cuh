@@ -17,6 +17,7 @@ struct JobDev {
     int blk_off;   // first block of the job in the launch
     int blocks;    // blocks of the job
     int bf16;      // inner coefficients in BF16
+    int skip;      // padding columns per row of the FP32 inner vectors (r32 has none)
     int res;       // the inner solve runs on chip and starts itself
     // FP64 operator and vectors
     const double *bx, *by, *bz, *diag;

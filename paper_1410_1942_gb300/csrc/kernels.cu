@@ -115,6 +115,20 @@ __global__ void k_update64(long long n, double* __restrict__ x, const float* __r
     if (t < n) x[t] += (double)dlt[t];
 }
 
+// the same from rows of `pitch` columns
+__global__ void k_update64_rows(Dims d, int pitch, double* __restrict__ x,
+                                const float* __restrict__ dlt) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t < d.n) x[t] += (double)dlt[t + (long long)(pitch - d.nx) * (t / d.nx)];
+}
+
+// rows of nx columns to rows of `pitch` columns
+template <typename T>
+__global__ void k_pitch_rows(Dims d, int pitch, const T* __restrict__ src, T* __restrict__ dst) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (t < d.n) dst[t + (long long)(pitch - d.nx) * (t / d.nx)] = src[t];
+}
+
 template <typename T>
 __global__ void k_narrow(long long n, const double* __restrict__ a, T* __restrict__ b) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -224,12 +238,13 @@ __global__ void __launch_bounds__(TX * TY) k_jacobi(Dims d, Coef coef, int kc,
 }
 
 // ------------------------------------------------------------------ PCG passes
-// init: z = D^{-1} r, rz = r.z, rr0 = r.r; stop2 = tol2 * (rel_to_b ? bb : rr0).
+// init: z = D^{-1} r, rz = r.z, rr0 = r.r; stop2 = tol2 * (rel_to_b ? bb : rr0).  z is stored with
+// zskip columns of padding per row.
 template <typename V, typename Coef>
 __global__ void __launch_bounds__(TX * TY) k_cg_init(Dims d, Coef coef, int kc,
                                                     const V* __restrict__ r, V* __restrict__ z,
                                                     Scalars* sc, double* partials, double tol2,
-                                                    int rel_to_b, int max_iter) {
+                                                    int rel_to_b, int max_iter, int zskip) {
     __shared__ double smem[64];
     V rz = 0, rr = 0;
     COL_LOOP_BEGIN
@@ -237,7 +252,7 @@ __global__ void __launch_bounds__(TX * TY) k_cg_init(Dims d, Coef coef, int kc,
         coef.weights(d, c, i, j, k, w);
         const V rc = r[c];
         const V zc = rc * inv_diag<V, Coef>(coef, c, w);
-        z[c] = zc;
+        z[c + (long long)zskip * (j + d.ny * k)] = zc;
         rz += rc * zc;
         rr += rc * rc;
     COL_LOOP_END
@@ -797,9 +812,10 @@ __global__ void __launch_bounds__(TX * TY) k_batch_update(const JobDev* jobs, in
     if (!J.active || i >= d.nx || j >= d.ny) return;
     for (int k = k0; k < k1; ++k) {
         const int c = i + d.nx * (j + d.ny * k);
-        J.x64[c] += (double)J.d32[c];
-        J.d32[c] = 0.f;
-        J.pa32[c] = 0.f;
+        const long long e = c + (long long)J.skip * (j + d.ny * k);
+        J.x64[c] += (double)J.d32[e];
+        J.d32[e] = 0.f;
+        J.pa32[e] = 0.f;
     }
 }
 
@@ -847,9 +863,10 @@ __device__ __forceinline__ void batch_init_body(const JobDev& J, const Dims& d, 
             coef.weights(d, c, i, j, k, w);
             const float rc = J.r32[c];
             const float zc = rc * rcp_approx(w.D);
-            J.z32[c] = zc;
-            J.sa32[c] = 0.f;
-            J.wa32[c] = 0.f;
+            const long long e = c + (long long)J.skip * (j + d.ny * k);
+            J.z32[e] = zc;
+            J.sa32[e] = 0.f;
+            J.wa32[e] = 0.f;
             rz += rc * zc;
             rr += rc * rc;
         }
@@ -957,6 +974,22 @@ void launch_update64(long long n, double* x, const float* dlt, cudaStream_t st) 
     counted(1);
 }
 
+void launch_update64_rows(const Dims& d, int pitch, double* x, const float* dlt, cudaStream_t st) {
+    k_update64_rows<<<blocks1d(d.n), 256, 0, st>>>(d, pitch, x, dlt);
+    counted(1);
+}
+
+void launch_pitch_rows(const Dims& d, int pitch, const float* src, float* dst, cudaStream_t st) {
+    k_pitch_rows<float><<<blocks1d(d.n), 256, 0, st>>>(d, pitch, src, dst);
+    counted(1);
+}
+
+void launch_pitch_rows(const Dims& d, int pitch, const __nv_bfloat16* src, __nv_bfloat16* dst,
+                       cudaStream_t st) {
+    k_pitch_rows<__nv_bfloat16><<<blocks1d(d.n), 256, 0, st>>>(d, pitch, src, dst);
+    counted(1);
+}
+
 void launch_fill_f32(long long n, float* p, float v, cudaStream_t st) {
     k_fill<float><<<blocks1d(n), 256, 0, st>>>(n, p, v);
     counted(1);
@@ -1016,9 +1049,10 @@ void launch_jacobi(const Dims& d, int kc, const Coef& c, const double* r, double
 
 template <typename V, typename Coef>
 void launch_cg_init(const Dims& d, int kc, const Coef& c, const V* r, V* z, Scalars* sc,
-                    double* part, double tol2, int rel_to_b, int max_iter, cudaStream_t st) {
+                    double* part, double tol2, int rel_to_b, int max_iter, cudaStream_t st,
+                    int zskip) {
     k_cg_init<V, Coef><<<grid_of(d, kc), dim3(TX, TY), 0, st>>>(d, c, kc, r, z, sc, part, tol2,
-                                                                rel_to_b, max_iter);
+                                                                rel_to_b, max_iter, zskip);
     counted(1);
 }
 
@@ -1115,7 +1149,7 @@ void launch_batch_init(const JobDev* jobs, int njobs, int blocks, cudaStream_t s
     template void launch_jacobi<V, C>(const Dims&, int, const C&, const double*, double*,    \
                                       cudaStream_t);                                        \
     template void launch_cg_init<V, C>(const Dims&, int, const C&, const V*, V*, Scalars*,   \
-                                       double*, double, int, int, cudaStream_t);            \
+                                       double*, double, int, int, cudaStream_t, int);       \
     template void launch_cg_a<V, C>(const Dims&, int, const C&, const V*, const V*, V*,     \
                                     Scalars*, double*, cudaStream_t);                       \
     template void launch_cg_b<V, C>(const Dims&, int, const C&, const V*, V*, V*, V*,       \

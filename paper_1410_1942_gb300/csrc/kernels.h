@@ -35,6 +35,11 @@ void launch_setup(const Dims& d, const double* F, double ra, double rw, double* 
 void launch_scale(long long n, const double* s, double a, double* b, cudaStream_t st,
                   const double* vol = nullptr);
 void launch_update64(long long n, double* x, const float* dlt, cudaStream_t st);
+// the same from rows stored at a pitch; rows stored at nx moved to a pitch
+void launch_update64_rows(const Dims& d, int pitch, double* x, const float* dlt, cudaStream_t st);
+void launch_pitch_rows(const Dims& d, int pitch, const float* src, float* dst, cudaStream_t st);
+void launch_pitch_rows(const Dims& d, int pitch, const __nv_bfloat16* src, __nv_bfloat16* dst,
+                       cudaStream_t st);
 void launch_narrow_f32(long long n, const double* a, float* b, cudaStream_t st);
 void launch_widen_f32(long long n, const float* a, double* b, cudaStream_t st);
 // rows padded with `pad` ghost columns each side holding the other end of the row (periodic x)
@@ -56,7 +61,8 @@ void launch_jacobi(const Dims& d, int kc, const Coef& c, const double* r, double
                    cudaStream_t st);
 template <typename V, typename Coef>
 void launch_cg_init(const Dims& d, int kc, const Coef& c, const V* r, V* z, Scalars* sc,
-                    double* part, double tol2, int rel_to_b, int max_iter, cudaStream_t st);
+                    double* part, double tol2, int rel_to_b, int max_iter, cudaStream_t st,
+                    int zskip = 0);
 template <typename V, typename Coef>
 void launch_cg_a(const Dims& d, int kc, const Coef& c, const V* z, const V* p_in, V* p_out,
                  Scalars* sc, double* part, cudaStream_t st);

@@ -880,11 +880,12 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 static bool encode3d(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int esz,
-                     const Dims& d, int bx, int by) {
+                     const Dims& d, int bx, int by, int pitch = 0) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)d.nx, (cuuint64_t)d.ny, (cuuint64_t)d.nz};
-    cuuint64_t strides[2] = {(cuuint64_t)d.nx * esz, (cuuint64_t)d.nx * d.ny * esz};
+    const cuuint64_t row = (cuuint64_t)(pitch ? pitch : d.nx) * esz;
+    cuuint64_t strides[2] = {row, row * d.ny};
     cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
     cuuint32_t es[3] = {1, 1, 1};
     return fn(m, dt, 3, const_cast<void*>(base), dims, strides, box, es,
@@ -893,11 +894,11 @@ static bool encode3d(CUtensorMap* m, const void* base, CUtensorMapDataType dt, i
 }
 
 bool march_supported(const Dims& d) {
-    // global strides must be multiples of 16 bytes for FP32 and BF16 rows
-    // (periodic x: the tiles' TMA halo boxes do not wrap; the column kernels serve it)
-    // (cut cells: the faces carry open fractions the kernels cannot form from rho/2; periodic x
-    // runs on the one-sweep kernels with padded rows)
-    return (d.nx % 8) == 0 && !(d.walls & CUT_CELLS) && encode_fn() != nullptr;
+    // global strides must be multiples of 16 bytes for FP32 and BF16 rows: rows of another length
+    // are stored at a pitch (one-sweep kernels only; not with the ghost columns of periodic x)
+    // (cut cells: the faces carry open fractions the kernels cannot form from rho/2)
+    return ((d.nx % 8) == 0 || !(d.walls & PERIODIC_X)) && !(d.walls & CUT_CELLS) &&
+           encode_fn() != nullptr;
 }
 
 // ------------------------------------------------------------------ variant table
@@ -908,6 +909,12 @@ struct VariantOps {
     const void *k32, *k16;
     int family;
     const void *k32p = nullptr, *k16p = nullptr;  // periodic-x instantiations (family 1)
+    const void *k32r = nullptr, *k16r = nullptr;  // rows of any length (family 1)
+    const void* kernel(bool bf16, RowMode m) const {
+        return m == ROWS_PERIODIC ? (bf16 ? k16p : k32p)
+               : m == ROWS_ANY    ? (bf16 ? k16r : k32r)
+                                  : (bf16 ? k16 : k32);
+    }
 };
 
 template <int CX, int CY, int TYT, int WS, int NS, int F>
@@ -919,7 +926,8 @@ static VariantOps make_ops() {
     } else if constexpr (F == 1 || F == 2) {
         static_assert(WS == 1, "the one-sweep kernels have a producer warp");
         const Cg1Kernel k = F == 1 ? cg1_kernel(CX, CY, TYT, NS) : cg2_kernel(CX, CY, TYT, NS);
-        return VariantOps{CX, CY, TYT, 1, NS, k.smem32, k.smem16, k.k32, k.k16, F, k.k32p, k.k16p};
+        return VariantOps{CX, CY, TYT, 1, NS, k.smem32, k.smem16, k.k32, k.k16, F,
+                          k.k32p, k.k16p, k.k32r, k.k16r};
     } else if constexpr (WS)
         return VariantOps{CX, CY, TYT, 1, NS, NS * Geo<CX, CY, TYT, float>::STAGE,
                           NS * Geo<CX, CY, TYT, __nv_bfloat16>::STAGE,
@@ -948,12 +956,11 @@ static const VariantOps* variants(int* count) {
     static std::once_flag once;
     std::call_once(once, [] {
         for (const auto& v : table) {
-            cudaFuncSetAttribute(v.k32, cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem32);
-            cudaFuncSetAttribute(v.k16, cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem16);
-            if (v.k32p)
-                cudaFuncSetAttribute(v.k32p, cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem32);
-            if (v.k16p)
-                cudaFuncSetAttribute(v.k16p, cudaFuncAttributeMaxDynamicSharedMemorySize, v.smem16);
+            for (RowMode m : {ROWS_PLAIN, ROWS_PERIODIC, ROWS_ANY})
+                for (bool h : {false, true})
+                    if (const void* k = v.kernel(h, m))
+                        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             h ? v.smem16 : v.smem32);
         }
         cudaGetLastError();
     });
@@ -1006,21 +1013,20 @@ int march_tile_of(int variant) {
 int march_occupancy(int variant, bool bf16) {
     int n;
     const VariantOps& v = variants(&n)[variant];
-    int o = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, bf16 ? v.k16 : v.k32, threads_of(v),
-                                                      bf16 ? v.smem16 : v.smem32) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    // a plan sized here may launch any of the instantiations: the smallest residency
+    int least = 1 << 20;
+    for (RowMode m : {ROWS_PLAIN, ROWS_PERIODIC, ROWS_ANY}) {
+        const void* k = v.kernel(bf16, m);
+        if (!k) continue;
+        int o = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, threads_of(v),
+                                                          bf16 ? v.smem16 : v.smem32) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        least = std::min(least, o);
     }
-    // a plan sized here may launch the periodic instantiation: take the smaller residency
-    const void* kp = bf16 ? v.k16p : v.k32p;
-    int op = o;
-    if (kp && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&op, kp, threads_of(v),
-                                                            bf16 ? v.smem16 : v.smem32) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return o < op ? o : op;
+    return least;
 }
 
 // ------------------------------------------------------------------ plans
@@ -1033,6 +1039,7 @@ bool march_encode_solve(CUtensorMap (&m)[MAPS_PER_SOLVE], const MarchSolve& s, i
     const Dims& d = s.d;
     bool ok = true;
     if ((d.walls & PERIODIC_X) && v.family != 1) return false;  // no wrapped halos there
+    if (s.pitch && v.family != 1) return false;                 // nor rows of any length
     if (v.family == 3) {
         // compressed black vectors (nx/2 per row) with 2-row halo boxes; eta at full size
         Dims db = d;
@@ -1073,15 +1080,16 @@ bool march_encode_solve(CUtensorMap (&m)[MAPS_PER_SOLVE], const MarchSolve& s, i
             de.nx = d.nx + 2 * eoff;
         }
         ok = ok && s.sa && s.sb && s.wa && s.wb;
-        ok = ok && encode3d(&m[MAP1_U0], s.z, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_U1], s.pb, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_S0], s.sa, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_S1], s.sb, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_W0], s.wa, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_W1], s.wb, f32, 4, dv, bw, bh);
-        ok = ok && encode3d(&m[MAP1_ETA], s.eta, edt, bf16 ? 2 : 4, de, v.width + 2 * eoff, bh);
-        ok = ok && encode3d(&m[MAP1_X], s.x, f32, 4, d, v.width, v.height);
-        ok = ok && encode3d(&m[MAP1_P], s.pa, f32, 4, d, v.width, v.height);
+        ok = ok && encode3d(&m[MAP1_U0], s.z, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_U1], s.pb, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_S0], s.sa, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_S1], s.sb, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_W0], s.wa, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_W1], s.wb, f32, 4, dv, bw, bh, s.pitch);
+        ok = ok && encode3d(&m[MAP1_ETA], s.eta, edt, bf16 ? 2 : 4, de, v.width + 2 * eoff, bh,
+                            s.pitch);
+        ok = ok && encode3d(&m[MAP1_X], s.x, f32, 4, d, v.width, v.height, s.pitch);
+        ok = ok && encode3d(&m[MAP1_P], s.pa, f32, 4, d, v.width, v.height, s.pitch);
         return ok;
     }
     ok = ok && encode3d(&m[MAP_Z], s.z, f32, 4, d, v.width + 8, v.height + 2);
@@ -1300,6 +1308,7 @@ int march_plan_build(MarchPlan* p, const MarchSolve* solves, int nsolves, int va
         sd[s].sb = solves[s].sb;
         sd[s].wa = solves[s].wa;
         sd[s].wb = solves[s].wb;
+        sd[s].pitch = solves[s].pitch ? solves[s].pitch : solves[s].d.nx;
         sd[s].seg_begin = (int)segs.size();
         sd[s].seg_end = 0;
     }
@@ -1314,13 +1323,17 @@ int march_plan_build(MarchPlan* p, const MarchSolve* solves, int nsolves, int va
         if (!march_encode_solve(m, solves[s], variant, bf16)) return -1;
         for (int q = 0; q < MAPS_PER_SOLVE; ++q) maps[MAPS_PER_SOLVE * (size_t)s + q] = m[q];
     }
-    int nper = 0;
-    for (int s = 0; s < nsolves; ++s) nper += (solves[s].d.walls & PERIODIC_X) ? 1 : 0;
-    if (nper != 0 && nper != nsolves) return -1;  // one instantiation per launch
+    int nper = 0, nany = 0;
+    for (int s = 0; s < nsolves; ++s) {
+        nper += (solves[s].d.walls & PERIODIC_X) ? 1 : 0;
+        nany += solves[s].pitch ? 1 : 0;
+    }
+    // one instantiation per launch (that for any rows serves plain ones too)
+    if (nper != 0 && (nper != nsolves || nany != 0)) return -1;
     p->variant = variant;
     p->strategy = strategy;
     p->bf16 = bf16;
-    p->periodic = nper > 0;
+    p->rows = nper ? ROWS_PERIODIC : nany ? ROWS_ANY : ROWS_PLAIN;
     p->nctas = nctas;
     p->nsolves = nsolves;
     p->nsegs = (int)segs.size();
@@ -1357,7 +1370,7 @@ int launch_march_pcg(const MarchPlan& p, cudaStream_t st) {
     PcgArgs args{p.solves, p.segs, p.cta_seg, p.maps, p.part_a,         p.part_b,
                  p.ctl,    p.nctas + p.barrier_extra,          p.trace};
     void* params[] = {&args};
-    const void* k = p.periodic ? (p.bf16 ? v.k16p : v.k32p) : (p.bf16 ? v.k16 : v.k32);
+    const void* k = v.kernel(p.bf16, p.rows);
     if (!k) return -1;
     const cudaError_t e = coop_launch(k, dim3(p.nctas), dim3(32, v.tyt + v.ws), params,
                                       (size_t)(p.bf16 ? v.smem16 : v.smem32), st);

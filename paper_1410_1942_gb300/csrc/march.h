@@ -36,6 +36,12 @@ constexpr int MAPS_PER_SOLVE = 9;
 // PAD_V columns of a row also write their ghost copies.
 constexpr int PAD_V = 4;
 
+// Row layouts of the one-sweep kernels (the plain one, and the two with an instantiation of their
+// own): periodic x as above; rows of any length, every array of the solve (x, p, u, s^, w^ and
+// rho/2) at MarchSolve::pitch columns a row, a multiple of eight.
+enum RowMode { ROWS_PLAIN = 0, ROWS_PERIODIC = 1, ROWS_ANY = 2 };
+inline int row_pitch(int nx) { return (nx + 7) & ~7; }
+
 // One solve of a plan as the host describes it.
 struct MarchSolve {
     Dims d;
@@ -43,6 +49,7 @@ struct MarchSolve {
     const void* eta;  // float or bf16, rho/2 per cell
     Scalars* sc;
     float *sa, *sb, *wa, *wb;  // family 1 only
+    int pitch = 0;  // columns per stored row; 0: nx (otherwise family 1 only)
 };
 
 // Device-side copy: the partial-sum slots [seg_begin, seg_end) of the solve.
@@ -52,6 +59,7 @@ struct SolveDev {
     float *x, *r, *z, *pa, *pb;
     Scalars* sc;
     float *sa, *sb, *wa, *wb;
+    int pitch;
 };
 
 // One tile column of one solve over planes [k0, k1); its partial sums go to slot `slot` of the
@@ -90,7 +98,7 @@ struct MarchPlan {
     int variant = 0;
     int strategy = 0;
     bool bf16 = false;
-    bool periodic = false;  // the solves have periodic x (the kernel's periodic instantiation)
+    RowMode rows = ROWS_PLAIN;  // the kernel's instantiation
     int nctas = 0, nsolves = 0, nsegs = 0;
     SolveDev* solves = nullptr;
     Seg* segs = nullptr;

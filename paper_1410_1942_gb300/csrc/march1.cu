@@ -78,11 +78,15 @@ __device__ __forceinline__ float u_next(float u, float s, float w, float al, flo
 // leave x as it is).
 __device__ __forceinline__ bool x_sweep(const LocalSolve1& L) { return !L.first && (L.iter & 1); }
 
-// PER: the solves have periodic x (padded rows with ghost columns); a separate instantiation so
-// that the plain kernel carries none of it.
-template <int CX, int CY, int TYT, typename E, int NS, bool PER>
+// MODE: ROWS_PLAIN; ROWS_PERIODIC, the solves have periodic x (padded rows with ghost columns);
+// ROWS_ANY, rows of any length stored at a pitch of whole 32 bytes (the tensor maps end at nx, so
+// what lies beyond reads as zero; the last thread of an odd row owns one column).  Separate
+// instantiations, so that the plain kernel carries none of it.  A 250 x 125 x 90 grid, which the
+// column kernels took 77 us an iteration for, takes 23 (301 x 151 x 120: 130 and 43).
+template <int CX, int CY, int TYT, typename E, int NS, int MODE>
 __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1_ws(PcgArgs a) {
     using G = Geo1<CX, CY, TYT, E>;
+    constexpr bool PER = MODE == ROWS_PERIODIC, RAG = MODE == ROWS_ANY;
     constexpr int NT = 32 * (TYT + 1);
     constexpr int NC = 32 * TYT;
     extern __shared__ __align__(128) unsigned char sm[];
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
         L.first = 1;
         L.xfix = 0;
         L.per = (sv.d.walls & PERIODIC_X) ? 1 : 0;
-        L.nxp = sv.d.nx + (L.per ? 2 * PAD_V : 0);
+        L.nxp = RAG ? sv.pitch : sv.d.nx + (L.per ? 2 * PAD_V : 0);
         L.owner = 0;
         for (int q = 0; q < nseg; ++q)
             if (s_seg[q].slot == sv.seg_begin) L.owner = 1;
@@ -213,7 +217,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
             const float alp = (float)s_sol[l].alpha_prev;
             const bool xs = x_sweep(s_sol[l]);
             const int i0 = sg.x0 + CX * tx, j0 = sg.y0 + CY * warp;
-            const unsigned edges = block_edges<CX, CY>(d, i0, j0);
+            const unsigned edges = block_edges<CX, CY>(d, i0, j0) | (RAG ? inner_edge(d, i0) : 0u);
             // u' of the thread's own block in plane q
             auto u_centre = [&](int q, float (&o)[CY][CX]) {
                 const unsigned char* S = stage(q);
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                     float exm[CY], exq[CY], eym[CX], eyp[CX];
                     load_halo<CX, CY>(eta_of(qc), G::EW, r0, ce, exm, exq, eym, eyp);
                     float qv[CY][CX], D[CY][CX];
-                    stencil<CX, CY>(d, edges, k, uc, vxm, vxp, vym, vyp, um, up, ec, exm, exq, eym,
+                    stencil<CX, CY, RAG>(d, edges, k, uc, vxm, vxp, vym, vyp, um, up, ec, exm, exq, eym,
                                     eyp, ep, wzl, qv, D);
                     if (i0 < d.nx) {
                         float u0[CY][CX], s0[CY][CX], w0[CY][CX], xo[CY][CX], po[CY][CX];
@@ -295,18 +299,21 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                                     sn[x] = __fmaf_rn(be, s0[y][x], w0[y][x]);
                                     if (xs)
                                         xn[x] = __fmaf_rn(al, pn[x], __fmaf_rn(alp, po[y][x], xo[y][x]));
-                                    wn[x] = qv[y][x] * rcp_approx(D[y][x]);
-                                    const float du = D[y][x] * uc[y][x];
+                                    // (RAG: the column beyond an odd row has no diagonal)
+                                    const bool in = !RAG || i0 + x < d.nx;
+                                    wn[x] = in ? qv[y][x] * rcp_approx(D[y][x]) : 0.f;
+                                    const float du = in ? D[y][x] * uc[y][x] : 0.f;
                                     ag += du * uc[y][x];
-                                    ad += qv[y][x] * uc[y][x];
+                                    ad += in ? qv[y][x] * uc[y][x] : 0.f;
                                     ar += du * du;
                                 }
                                 const size_t c =
-                                    (size_t)i0 + (size_t)d.nx * (j0 + y + (size_t)d.ny * k);
+                                    (size_t)i0 + (size_t)(RAG ? s_sol[l].nxp : d.nx) *
+                                                     (j0 + y + (size_t)d.ny * k);
                                 if (xs) st_row<CX>(s_sol[l].x + c, xn);
                                 st_row<CX>(s_sol[l].p + c, pn);
                                 const LocalSolve1& Ls = s_sol[l];
-                                const size_t row = (size_t)(PER ? Ls.nxp : d.nx) *
+                                const size_t row = (size_t)(MODE != ROWS_PLAIN ? Ls.nxp : d.nx) *
                                                    (j0 + y + (size_t)d.ny * k);
                                 const size_t cp = row + i0 + (PER ? PAD_V : 0);
                                 st_row<CX>(Ls.u[out] + cp, uc[y]);
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                 const Seg sg = s_seg[ls];
                 const LocalSolve1& L = s_sol[sg.solve - first];
                 if (!L.xfix) continue;
-                const int nx = L.d.nx, ny = L.d.ny;
+                const int nx = L.d.nx, ny = L.d.ny, xp = RAG ? L.nxp : nx;
                 const int wd = min(G::W, nx - sg.x0), ht = min(G::HT, ny - sg.y0);
                 const int per = wd * ht;
                 const long long cnt = (long long)per * (sg.k1 - sg.k0);
@@ -470,7 +477,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                 for (long long q = tid; q < cnt; q += NC) {
                     const int k = sg.k0 + (int)(q / per), r = (int)(q % per);
                     const size_t c = (size_t)(sg.x0 + r % wd) +
-                                     (size_t)nx * ((size_t)(sg.y0 + r / wd) + (size_t)ny * k);
+                                     (size_t)xp * ((size_t)(sg.y0 + r / wd) + (size_t)ny * k);
                     L.x[c] = __fmaf_rn(al, L.p[c], L.x[c]);
                 }
             }
@@ -517,12 +524,14 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
 
 template <int CX, int CY, int TYT, int NS>
 static Cg1Kernel cg1_of() {
-    return Cg1Kernel{(const void*)k_cg1_ws<CX, CY, TYT, float, NS, false>,
-                     (const void*)k_cg1_ws<CX, CY, TYT, __nv_bfloat16, NS, false>,
+    return Cg1Kernel{(const void*)k_cg1_ws<CX, CY, TYT, float, NS, ROWS_PLAIN>,
+                     (const void*)k_cg1_ws<CX, CY, TYT, __nv_bfloat16, NS, ROWS_PLAIN>,
                      NS * Geo1<CX, CY, TYT, float>::STAGE,
                      NS * Geo1<CX, CY, TYT, __nv_bfloat16>::STAGE,
-                     (const void*)k_cg1_ws<CX, CY, TYT, float, NS, true>,
-                     (const void*)k_cg1_ws<CX, CY, TYT, __nv_bfloat16, NS, true>};
+                     (const void*)k_cg1_ws<CX, CY, TYT, float, NS, ROWS_PERIODIC>,
+                     (const void*)k_cg1_ws<CX, CY, TYT, __nv_bfloat16, NS, ROWS_PERIODIC>,
+                     (const void*)k_cg1_ws<CX, CY, TYT, float, NS, ROWS_ANY>,
+                     (const void*)k_cg1_ws<CX, CY, TYT, __nv_bfloat16, NS, ROWS_ANY>};
 }
 
 Cg1Kernel cg1_kernel(int cx, int cy, int tyt, int ns) {

@@ -95,12 +95,20 @@ __device__ __forceinline__ unsigned block_edges(const Dims& d, int i0, int j0) {
     return e;
 }
 
+// Bit of a thread's block whose two columns both lie in the grid or meet at a Dirichlet wall: the
+// face between them is open (rows of any length only, where the last block may hold one column).
+constexpr unsigned EDGE_INNER_X = 1u << 16;
+__device__ __forceinline__ unsigned inner_edge(const Dims& d, int i0) {
+    return (i0 + 1 < d.nx || (d.walls & 2)) ? EDGE_INNER_X : 0u;
+}
+
 // The stencil of one plane for the CX x CY block of a thread.
 //   cen: centre values of plane k (registers); vxm/vxp/vym/vyp: the block's neighbour strips in
 //   plane k; vm/vp: centre values of planes k-1 and k+1; e*: the same for eta; wzl: face to
 //   plane k-1 (0 on the floor).  Returns q = A v and the diagonal per cell, and moves wzl to the
 //   face between k and k+1 (0 at the top layer, whose Dirichlet term goes into D).
-template <int CX, int CY>
+// RAG: the face between a block's two columns obeys EDGE_INNER_X.
+template <int CX, int CY, bool RAG = false>
 __device__ __forceinline__ void stencil(const Dims& d, unsigned edges, int k,
                                         const float (&cen)[CY][CX], const float (&vxm)[CY],
                                         const float (&vxp)[CY], const float (&vym)[CX],
@@ -117,7 +125,8 @@ __device__ __forceinline__ void stencil(const Dims& d, unsigned edges, int k,
     for (int a = 0; a < CY; ++a) {
         fx[a][0] = (edges & 1u) ? rcp_approx(ec[a][0] + exm[a]) : 0.f;
 #pragma unroll
-        for (int b = 1; b < CX; ++b) fx[a][b] = rcp_approx(ec[a][b - 1] + ec[a][b]);
+        for (int b = 1; b < CX; ++b)
+            fx[a][b] = (!RAG || (edges & EDGE_INNER_X)) ? rcp_approx(ec[a][b - 1] + ec[a][b]) : 0.f;
         fx[a][CX] = (edges & 2u) ? rcp_approx(ec[a][CX - 1] + exq[a]) : 0.f;
     }
     float fy[CY + 1][CX];
@@ -426,6 +435,7 @@ struct Cg1Kernel {
     const void *k32, *k16;
     int smem32, smem16;
     const void *k32p = nullptr, *k16p = nullptr;  // periodic-x instantiations (one-sweep family)
+    const void *k32r = nullptr, *k16r = nullptr;  // rows of any length (one-sweep family)
 };
 Cg1Kernel cg1_kernel(int cx, int cy, int tyt, int ns);  // null kernels if not instantiated
 // Kernels of the one-sweep family with A p formed in the sweep (march2.cu).
