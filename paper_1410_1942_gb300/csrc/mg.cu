@@ -709,7 +709,7 @@ struct BodyCgB {
             for (int b = 0; b < 2; ++b) {
                 xn.v[a][b] = X[0].v[a][b] + alpha * u.v[a][b];
                 rn.v[a][b] = X[1].v[a][b] - alpha * q.v[a][b];
-                zn.v[a][b] = omega * rn.v[a][b] / D.v[a][b];
+                zn.v[a][b] = div_refined(omega * rn.v[a][b], D.v[a][b]);
                 rr += rn.v[a][b] * rn.v[a][b];
             }
         st2(x, c, xn.v[0][0], xn.v[0][1]);
@@ -763,7 +763,7 @@ struct BodySmooth {
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                yn.v[a][b] = u.v[a][b] + omega * (X[0].v[a][b] - q.v[a][b]) / D.v[a][b];
+                yn.v[a][b] = u.v[a][b] + div_refined(omega * (X[0].v[a][b] - q.v[a][b]), D.v[a][b]);
                 rz += X[0].v[a][b] * yn.v[a][b];
             }
         st2(y, c, yn.v[0][0], yn.v[0][1]);
