@@ -678,6 +678,11 @@ extern "C" int poisson_create(int nx, int ny, int nz, double h, const poisson_op
     if (o.precond == POISSON_MG && rc == POISSON_OK) {
         mg_plan(H->d, &H->mg);
         A(mg_alloc(&H->mg, o.precision == POISSON_FP64));
+        const bool bf16 = o.precision == POISSON_FP32_BF16COEF;
+        if (rc == POISSON_OK && o.precision != POISSON_FP64 && fine_maps_fit(H->d) &&
+            fine_maps_build(&H->fine, H->d, bf16 ? (const void*)H->eta16 : (const void*)H->eta32, bf16,
+                            H->z32, H->p32a, H->p32b, (const float*)H->mg.x[0], H->r32, H->d32))
+            H->mg.fine = &H->fine;
     }
     if (rc == POISSON_OK && lib_malloc_host((void**)&H->sc_host, 2 * sizeof(Scalars)) != cudaSuccess) {
         cudaGetLastError();
@@ -831,6 +836,7 @@ extern "C" int poisson_set_apertures(poisson_t* H, const double* ax, const doubl
             *q = nullptr;
         }
         H->d.walls &= ~CUT_CELLS;
+        if (H->fine.on) H->mg.fine = &H->fine;
         // the plan built at create, if any
         H->march = H->plan.segs != nullptr && H->opts.precond == POISSON_JACOBI;
         H->rb = H->plan.segs != nullptr && H->opts.precond == POISSON_RBSSOR;
@@ -860,6 +866,7 @@ extern "C" int poisson_set_apertures(poisson_t* H, const double* ax, const doubl
     CK(copy_user(H->vol64, vol, sizeof(double) * n, kind, H->st));
     CK(cudaStreamSynchronize(H->st));
     H->d.walls |= CUT_CELLS;
+    H->mg.fine = nullptr;
     H->march = false;  // the marching kernels form faces from rho/2 and cannot carry fractions
     H->rb = false;
     H->ready = false;  // poisson_set_density builds the cut operator
@@ -1026,6 +1033,9 @@ static int cg_loop_columns(poisson_t* H, const Coef& coef, V* x, V* r, V* z, V* 
     const int kc = H->kc;
     cudaStream_t st = H->st;
     auto A = [=](bool in_a) {
+        if constexpr (is_coef_eta<Coef>::value)
+            if (H->mg.fine)
+                return launch_fine_a(H->fine, d, in_a, in_a ? pb : pa, H->sc, H->partials, st);
         launch_cg_a<V, Coef>(d, kc, coef, z, in_a ? pa : pb, in_a ? pb : pa, H->sc, H->partials, st);
     };
     const bool ssor = H->opts.precond == POISSON_RBSSOR;

@@ -10,6 +10,7 @@
 #include "internal.cuh"
 #include "march.h"
 #include "mg.h"
+#include "mg_tma.h"
 #include "resident.h"
 
 struct poisson_s {
@@ -71,6 +72,7 @@ struct poisson_s {
     float* io_c32 = nullptr;  // SSOR apply scratch (FP32)
     // multigrid V-cycle hierarchy (POISSON_MG): Galerkin levels in the inner precision
     pcg::MgHier mg{};
+    pcg::FineMaps fine{};  // tensor maps of the fine passes (in use while mg.fine points here)
     // TMA plane-marching kernels for the FP32 inner solve (when the shape allows them)
     bool march = false;
     // red-black SSOR (omega = 1) inner solve on the plane-marching kernels of march_rb.cu: CG on

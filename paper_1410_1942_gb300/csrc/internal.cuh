@@ -60,6 +60,27 @@ struct Scalars {
 
 enum Done { RUNNING = 0, CONVERGED = 1, BREAKDOWN = 2, CAPPED = 3, TIMEDOUT = 4 };
 
+// The (r, z) of a new iterate of the preconditioned loops: stored after the start (mode 0), else the
+// iteration is counted and beta or the stopping state set.
+__device__ __forceinline__ void cg_next(Scalars* sc, double rz_new, int mode) {
+    if (mode == 0) {
+        sc->rz = rz_new;
+        if (!isfinite(rz_new) || !(rz_new > 0.0)) sc->done = BREAKDOWN;
+    } else {
+        sc->iter += 1;
+        if (!isfinite(rz_new) || rz_new < 0.0 || !isfinite(sc->rr)) {
+            sc->done = BREAKDOWN;
+        } else if (sc->rr <= sc->stop2) {
+            sc->done = CONVERGED;
+        } else if (sc->iter >= sc->max_iter) {
+            sc->done = CAPPED;
+        } else {
+            sc->beta = rz_new / sc->rz;
+            sc->rz = rz_new;
+        }
+    }
+}
+
 // Hardware reciprocal (MUFU), flush-to-zero: deterministic for a given input.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;

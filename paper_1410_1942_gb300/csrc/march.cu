@@ -893,6 +893,11 @@ static bool encode3d(CUtensorMap* m, const void* base, CUtensorMapDataType dt, i
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool march_encode_box(CUtensorMap* m, const void* base, bool half, const Dims& d, int bx, int by) {
+    return encode3d(m, base, half ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                    half ? 2 : 4, d, bx, by);
+}
+
 bool march_supported(const Dims& d) {
     // global strides must be multiples of 16 bytes for FP32 and BF16 rows: rows of another length
     // are stored at a pitch (one-sweep kernels only; not with the ghost columns of periodic x)

@@ -137,6 +137,8 @@ struct PcgArgs {
 enum { TR_A = 0, TR_BAR1, TR_ALPHA, TR_B, TR_BAR2, TR_BETA, TR_ITERS, TR_IMB, TR_REL, TR_SUM,
        TR_DECIDE, TRACE_PARTS };
 
+// Tensor map of a grid's array (float, or bf16 when half) with boxes of bx x by cells of one plane.
+bool march_encode_box(CUtensorMap* m, const void* base, bool half, const Dims& d, int bx, int by);
 bool march_supported(const Dims& d);
 int march_variant_count();
 MarchVariant march_variant(int id);

@@ -13,6 +13,7 @@
 #include "poisson.h"
 #include "mg.h"
 #include "kernels.h"
+#include "mg_tma.h"
 #include "plane_tile.cuh"
 
 namespace pcg {
@@ -428,25 +429,7 @@ __device__ __forceinline__ void reduce_rz(V rz, Scalars* sc, double* partials, d
                                           int mode) {
     double v[1] = {(double)rz}, tot[1];
     if (grid_sum<1>(v, partials, &sc->ticket, tot, smem)) {
-        if (threadIdx.x == 0 && threadIdx.y == 0) {
-            const double rz_new = tot[0];
-            if (mode == 0) {
-                sc->rz = rz_new;
-                if (!isfinite(rz_new) || !(rz_new > 0.0)) sc->done = BREAKDOWN;
-            } else {
-                sc->iter += 1;
-                if (!isfinite(rz_new) || rz_new < 0.0 || !isfinite(sc->rr)) {
-                    sc->done = BREAKDOWN;
-                } else if (sc->rr <= sc->stop2) {
-                    sc->done = CONVERGED;
-                } else if (sc->iter >= sc->max_iter) {
-                    sc->done = CAPPED;
-                } else {
-                    sc->beta = rz_new / sc->rz;
-                    sc->rz = rz_new;
-                }
-            }
-        }
+        if (threadIdx.x == 0 && threadIdx.y == 0) cg_next(sc, tot[0], mode);
     }
 }
 
@@ -1082,6 +1065,9 @@ __global__ void __launch_bounds__(TX * TY) k_mg_cg_b(Dims d, Coef coef, int kc,
     }
 }
 
+// Whether the fine passes run on TMA-staged planes (the handle's maps are for this residual).
+inline bool fine_of(const MgHier& m, const float* r) { return m.fine && m.fine->r == r; }
+
 // z = V_0(r) given x[0] = w D^-1 r: restrictions down, the coarsest sweeps, prolongation +
 // post-smoothing up; the fine smoothing writes z (and reduces r.z when mode >= 0).
 template <typename V, typename Coef>
@@ -1110,6 +1096,11 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
             }
         }
         if constexpr (is_coef_eta<Coef>::value) {
+            if (l == 0 && fine_of(*m, r)) {
+                launch_fine_restrict(*m->fine, df, dc, f[2], (const float*)m->diag[1],
+                                     (float*)m->r[1], (float*)m->x[1], om, sc, st);
+                done = true;
+            }
             if (!done && l == 0 && quad_tiles_fit(df)) {
                 launch_pdl(k_mg_restrict_q<EtaOf<Coef>>, quad_grid(df, quad_kc(df, QB_RESTRICT)),
                            dim3(TX, TY), 0, st, df, coef, quad_kc(df, QB_RESTRICT), r, (const V*)m->x[0], dc, f[2], (const V*)m->diag[1],
@@ -1174,7 +1165,10 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
     }
     const int* f = m->f[0];
     if constexpr (is_coef_eta<Coef>::value) {
-        if (quad_tiles_fit(d))
+        if (fine_of(*m, r))
+            launch_fine_smooth(*m->fine, d, m->d[1], f[2] - 1, (const float*)m->y[1], al, om, z, sc,
+                               part, mode, st);
+        else if (quad_tiles_fit(d))
             launch_pdl(k_mg_smooth_q<EtaOf<Coef>>, quad_grid(d, quad_kc(d, QB_SMOOTH)), dim3(TX, TY),
                        0, st, d, coef, quad_kc(d, QB_SMOOTH), r, (const V*)m->x[0], (const V*)m->y[1], m->d[1], f[2] - 1,
                 al, om, z, sc, part, mode);
@@ -1301,7 +1295,10 @@ template <typename V, typename Coef>
 void mg_cg_b(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* p, V* x, V* r, V* z,
              Scalars* sc, double* part, cudaStream_t st) {
     if constexpr (is_coef_eta<Coef>::value) {
-        if (quad_tiles_fit(d))
+        if (fine_of(*m, r))
+            launch_fine_b(*m->fine, d, p == m->fine->pa, x, r, (float*)m->x[0], (float)MG_OMEGA, sc,
+                          part, st);
+        else if (quad_tiles_fit(d))
             launch_pdl(k_mg_cg_b_q<EtaOf<Coef>>, quad_grid(d, quad_kc(d, QB_CG_B)), dim3(TX, TY), 0,
                        st, d, coef, quad_kc(d, QB_CG_B), p, x, r, (V*)m->x[0], (V)MG_OMEGA, sc, part);
         else if (plane_tiles_fit(d))

@@ -29,7 +29,10 @@ constexpr double MG_ALPHA = 1.5;   // coarse-correction scaling
 constexpr int MG_COARSE_MAX = 512;
 constexpr int MG_COARSE_SWEEPS = 16;
 
+struct FineMaps;
+
 struct MgHier {
+    const FineMaps* fine = nullptr;  // the fine passes on TMA-staged planes (mg_tma.h), or null
     int nlev = 0;     // levels, the fine one included (>= 2 once planned)
     bool dbl = false;  // level arrays in FP64 (FP64 handles) or FP32
     Dims d[MG_MAX_LEVELS] = {};
