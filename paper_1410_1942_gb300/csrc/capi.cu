@@ -896,20 +896,29 @@ static void prof_add(poisson_t* H, int cls, cudaEvent_t a, cudaEvent_t b) {
 // ------------------------------------------------------------------ inner CG loop
 // Queues chunks of CG_CHUNK iterations; reads the scalars of chunk n while chunk n+1 runs.
 // pass_a(p_in_is_a) and pass_b(p_is_a) launch one CG phase each on the handle's stream.
-// A stream that can be captured into a graph (not the legacy or per-thread default stream).
-static bool capturable(cudaStream_t st) {
-    return st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread;
-}
-
-// Captures `passes` (the launches of one CG chunk) on the handle's stream as a graph for code
-// path `tag`.  The passes' launch arguments (buffers, scalars, sizes) are the handle's own and do
-// not change between chunks, and a chunk has an even number of iterations, so every chunk starts
-// on the same p buffer and one graph serves them all.  false (nothing launched, no graph) when
-// the capture fails; the caller then launches the passes directly.
+// Captures `passes` (the launches of one CG chunk) as a graph for code path `tag`, on a stream made
+// for it (the handle's own may be the legacy default stream, which cannot be captured but takes
+// graph launches); the passes launch on the handle's current stream.  Their launch arguments
+// (buffers, scalars, sizes) are the handle's own and do not change between chunks, and a chunk has
+// an even number of iterations, so every chunk starts on the same p buffer and one graph serves them
+// all.  false (nothing launched, no graph) when the capture fails; the caller then launches the
+// passes directly.
 template <typename F>
 static bool capture_chunk(poisson_t* H, const void* tag, F&& passes) {
     drop_chunk_graph(H);
-    if (cudaStreamBeginCapture(H->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    struct Swap {  // H->st is the capture stream while this lives
+        poisson_t* h;
+        cudaStream_t own, cap = nullptr;
+        explicit Swap(poisson_t* p) : h(p), own(p->st) {
+            if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) cap = nullptr;
+            if (cap) h->st = cap;
+        }
+        ~Swap() {
+            h->st = own;
+            if (cap) cudaStreamDestroy(cap);
+        }
+    } swap(H);
+    if (!swap.cap || cudaStreamBeginCapture(H->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -939,7 +948,10 @@ static bool capture_chunk(poisson_t* H, const void* tag, F&& passes) {
 template <typename V, typename Coef, typename PassA, typename PassB>
 static int cg_loop(poisson_t* H, const Coef& coef, V* r, V* z, double tol2, int rel_to_b,
                    int max_iter, Scalars* result, PassA pass_a, PassB pass_b) {
-    const int K = CG_CHUNK;
+    // Iterations queued per look at the scalars, with the next chunk queued behind: a solve runs
+    // up to two chunks too many, every kernel of which only looks at the state.  A V-cycle's
+    // eleven launches make that dear (half a chunk of eight was 8 % of a 256x128x128 solve).
+    const int K = H->opts.precond == POISSON_MG ? MG_CHUNK : CG_CHUNK;
     cudaStream_t st = H->st;
     const bool prof = H->prof_on;
     if (H->opts.precond == POISSON_MG)
@@ -951,7 +963,8 @@ static int cg_loop(poisson_t* H, const Coef& coef, V* r, V* z, double tol2, int 
     else
         launch_cg_init<V, Coef>(H->d, H->kc, coef, r, z, H->sc, H->partials, tol2, rel_to_b,
                                 max_iter, st);
-    static_assert(CG_CHUNK % 2 == 0, "a chunk returns to the p buffer it started from");
+    static_assert(CG_CHUNK % 2 == 0 && MG_CHUNK % 2 == 0,
+                  "a chunk returns to the p buffer it started from");
     static const char tag = 0;  // this code path (one per instantiation of the loop)
     bool in_is_a = true;
     auto passes = [&] {
@@ -964,9 +977,9 @@ static int cg_loop(poisson_t* H, const Coef& coef, V* r, V* z, double tol2, int 
     };
     auto enqueue_chunk = [&](int slot) -> int {
         cudaEvent_t* ev = prof ? &H->prof_ev[slot * PROF_PER_CHUNK] : nullptr;
-        // without per-phase events, on a capturable stream: one graph launch per chunk
-        if (!prof && capturable(st) &&
-            (H->chunk_tag == &tag || capture_chunk(H, &tag, passes))) {
+        // without per-phase events: one graph launch per chunk (a small V-cycle launch by launch is
+        // bound by the host: 58 us an iteration at 64x48x32)
+        if (!prof && (H->chunk_tag == &tag || capture_chunk(H, &tag, passes))) {
             CK(cudaGraphLaunch(H->chunk_exec, st));
             g_kernel_launches.fetch_add((unsigned long long)H->chunk_nodes,
                                         std::memory_order_relaxed);
@@ -1031,8 +1044,9 @@ static int cg_loop_columns(poisson_t* H, const Coef& coef, V* x, V* r, V* z, V* 
                            double tol2, int rel_to_b, int max_iter, Scalars* result) {
     const Dims d = H->d;
     const int kc = H->kc;
-    cudaStream_t st = H->st;
+    // (the stream is looked up at each launch: a capture swaps it)
     auto A = [=](bool in_a) {
+        cudaStream_t st = H->st;
         if constexpr (is_coef_eta<Coef>::value)
             if (H->mg.fine)
                 return launch_fine_a(H->fine, d, in_a, in_a ? pb : pa, H->sc, H->partials, st);
@@ -1042,6 +1056,7 @@ static int cg_loop_columns(poisson_t* H, const Coef& coef, V* x, V* r, V* z, V* 
     const bool mg = H->opts.precond == POISSON_MG;
     const double omega = H->opts.omega;
     auto B = [=](bool p_a) {
+        cudaStream_t st = H->st;
         if (mg)
             mg_cg_b<V, Coef>(&H->mg, d, kc, coef, p_a ? pa : pb, x, r, z, H->sc, H->partials, st);
         else if (ssor)

@@ -88,7 +88,7 @@ struct poisson_s {
     pcg::MarchPlan plan{};  // persistent work-list launch over this handle's grid
     pcg::MarchCtl* ctl_host = nullptr;  // pinned staging of plan.ctl
     // the column-kernel CG chunk (CG_CHUNK iterations of phases A and B) as a CUDA graph,
-    // captured on the first chunk run on a capturable stream; chunk_tag names the code path it
+    // captured on the first chunk; chunk_tag names the code path it
     // was captured for, chunk_nodes its kernels
     cudaGraph_t chunk_graph = nullptr;
     cudaGraphExec_t chunk_exec = nullptr;
@@ -101,6 +101,7 @@ struct poisson_s {
 };
 
 constexpr int CG_CHUNK = 8;                    // CG iterations queued per host check
+constexpr int MG_CHUNK = 2;                    // ... with the V-cycle
 constexpr int PROF_PER_CHUNK = 3 * CG_CHUNK;   // events per chunk slot when profiling
 constexpr int PROF_RES = 2 * PROF_PER_CHUNK;   // event pair around a residual kernel
 constexpr int PROF_PCG = PROF_RES + 2;         // event pair around a persistent PCG launch
