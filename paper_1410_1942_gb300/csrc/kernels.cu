@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 
 namespace pcg {
 
@@ -29,71 +30,156 @@ __device__ __forceinline__ double rho_of(double F, double ra, double rw) {
     return __dadd_rn(ra, __dmul_rn(F, __dadd_rn(rw, -ra)));
 }
 
+// Unsigned division by an invariant divisor by a multiplication and a shift (Granlund and
+// Montgomery, "Division by Invariant Integers using Multiplication", 1994), for n < 2^31.
+struct FastDiv {
+    unsigned m, s;
+    explicit FastDiv(int d) {
+        s = 0;
+        while ((1ll << s) < d) ++s;
+        m = (unsigned)((((1ull << s) - (unsigned long long)d) << 32) / (unsigned long long)d + 1);
+    }
+    __device__ __forceinline__ int div(int n) const {
+        return (int)((__umulhi((unsigned)n, m) + (unsigned)n) >> s);
+    }
+};
+
+// What the operator needs of cells that are all air (F = 0) or all water (F = 1), worked out once
+// on the host by the same rounded expressions as the kernel's.
+struct Phases {
+    double face[3];            // 2/(rho_a + rho_b) of air-air, air-water, water-water faces
+    double wall[2];            // 2/rho
+    double diag[2], dinv[2];   // six equal faces summed in the kernel's order, and the inverse
+    float eta[2];              // rho/2
+    int ok;                    // both densities are positive and finite
+};
+
+static Phases phases_of(double ra, double rw) {
+    Phases p{};
+    const double step = rw - ra, rho[2] = {ra, ra + step};
+    p.ok = std::isfinite(step);
+    for (int q = 0; q < 2; ++q) {
+        p.ok = p.ok && rho[q] > 0.0 && std::isfinite(rho[q]);
+        const double f = 2.0 / (rho[q] + rho[q]);
+        p.face[2 * q] = f;
+        p.wall[q] = 2.0 / rho[q];
+        volatile double s = f + f;  // (each sum rounded to double)
+        for (int a = 0; a < 4; ++a) s = s + f;
+        p.diag[q] = s;
+        p.dinv[q] = 1.0 / s;
+        p.eta[q] = (float)(0.5 * rho[q]);
+    }
+    p.face[1] = 2.0 / (rho[0] + rho[1]);
+    return p;
+}
+
+// 0: all air, 1: all water, 2: neither
+__device__ __forceinline__ int phase_of(double F) {
+    const long long b = __double_as_longlong(F);
+    return b == 0 ? 0 : b == 0x3ff0000000000000ll ? 1 : 2;
+}
+
+// The operator from F, one cell a thread: its three low faces, its diagonal and rho/2.
+// diag = low faces x, y, z, then high faces x, y, z (2/rho_c on the top layer) (+ 2/rho_c for each
+// Dirichlet side/bottom wall the cell touches, x-, x+, y-, y+, z-), summed in that order;
+// top[i + nx j] = 2/rho_c of the top layer; rinv2[c] = 2/rho_c (only with Dirichlet walls).
 // bad: set to 1 when some cell's density is not a positive finite number (F non-finite, or so
-// far outside [0, 1] that rho <= 0): the operator is then not SPD
-__global__ void k_setup_faces(Dims d, const double* __restrict__ F, double ra, double rw,
-                              double* __restrict__ bx, double* __restrict__ by,
-                              double* __restrict__ bz, float* __restrict__ eta32,
-                              __nv_bfloat16* __restrict__ eta16, Apertures ap,
-                              unsigned* __restrict__ bad) {
+// far outside [0, 1] that rho <= 0): the operator is then not SPD.
+//
+// Bound by the FP64 pipe (two operations a clock and SM) wherever it divides: three divisions a
+// face pass and two a diagonal pass took 301 and 127 us on 256x128x128, against 30 us for the
+// bytes.  Nearly every cell and all its neighbours are of one phase, so a face between cells of
+// pure phase takes one of three values worked out once, and a cell in the middle of one phase
+// none of the sums either; only cells at the interface and the boundary compute, by the same
+// expressions bit for bit.  A cell works out its three high faces again instead of reading them
+// from a first pass.  256x128x128 with a wavy surface (5 % of the warps divide): 92 us.
+__global__ void __launch_bounds__(256) k_setup(Dims d, FastDiv by_nx, FastDiv by_ny,
+                                               const double* __restrict__ F, double ra, double rw,
+                                               const __grid_constant__ Phases ph,
+                                               double* __restrict__ bx, double* __restrict__ by,
+                                               double* __restrict__ bz, double* __restrict__ diag,
+                                               double* __restrict__ dinv, double* __restrict__ top,
+                                               double* __restrict__ rinv2, float* __restrict__ eta32,
+                                               __nv_bfloat16* __restrict__ eta16, Apertures ap,
+                                               unsigned* __restrict__ bad) {
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (tid >= d.n) return;
     const int c = (int)tid;
-    const int i = c % d.nx, j = (c / d.nx) % d.ny, k = c / d.sxy;
-    const double rc = rho_of(F[c], ra, rw);
-    if (!(rc > 0.0) || !isfinite(rc)) *bad = 1u;
-    // periodic x: the low face of cell 0 couples it to cell nx-1 of its row
-    bx[c] = (i > 0 || (d.walls & PERIODIC_X))
-                ? 2.0 / __dadd_rn(rc, rho_of(F[i > 0 ? c - 1 : c + d.nx - 1], ra, rw))
-                : 0.0;
-    by[c] = (j > 0) ? 2.0 / __dadd_rn(rc, rho_of(F[c - d.nx], ra, rw)) : 0.0;
-    bz[c] = (k > 0) ? 2.0 / __dadd_rn(rc, rho_of(F[c - d.sxy], ra, rw)) : 0.0;
-    if (ap.ax) {
-        // cut cells: each face scaled by its open fraction; closed next to a cell with no fluid
-        const long long fu = i + (long long)(d.nx + 1) * (j + (long long)d.ny * k);
-        const long long fv = i + (long long)d.nx * (j + (long long)(d.ny + 1) * k);
-        const bool act = ap.vol[c] > 0.0;
-        const int cxm = i > 0 ? c - 1 : c + d.nx - 1;
-        bx[c] = (act && ap.vol[cxm] > 0.0) ? __dmul_rn(ap.ax[fu], bx[c]) : 0.0;
-        by[c] = (act && j > 0 && ap.vol[c - d.nx] > 0.0) ? __dmul_rn(ap.ay[fv], by[c]) : 0.0;
-        bz[c] = (act && k > 0 && ap.vol[c - d.sxy] > 0.0) ? __dmul_rn(ap.az[c], bz[c]) : 0.0;
+    const int row = by_nx.div(c), k = by_ny.div(row);
+    const int i = c - row * d.nx, j = row - k * d.ny;
+    const bool per = (d.walls & PERIODIC_X) != 0;
+    // neighbours; periodic x: the low face of cell 0 couples it to cell nx-1 of its row
+    const bool hx0 = i > 0 || per, hx1 = i + 1 < d.nx || per;
+    const bool hy0 = j > 0, hy1 = j + 1 < d.ny, hz0 = k > 0, hz1 = k + 1 < d.nz;
+    const int x0 = i > 0 ? c - 1 : c + d.nx - 1, x1 = i + 1 < d.nx ? c + 1 : c + 1 - d.nx;
+    const double Fc = F[c];
+    const double Fx0 = hx0 ? F[x0] : Fc, Fx1 = hx1 ? F[x1] : Fc;
+    const double Fy0 = hy0 ? F[c - d.nx] : Fc, Fy1 = hy1 ? F[c + d.nx] : Fc;
+    const double Fz0 = hz0 ? F[c - d.sxy] : Fc, Fz1 = hz1 ? F[c + d.sxy] : Fc;
+    const int pc = ph.ok ? phase_of(Fc) : 2;
+    const bool full = hx0 && hx1 && hy0 && hy1 && hz0 && hz1 && !ap.vol;
+    if (full && pc < 2 && Fx0 == Fc && Fx1 == Fc && Fy0 == Fc && Fy1 == Fc && Fz0 == Fc && Fz1 == Fc) {
+        const double f = pc ? ph.face[2] : ph.face[0];
+        bx[c] = f;
+        by[c] = f;
+        bz[c] = f;
+        diag[c] = pc ? ph.diag[1] : ph.diag[0];
+        if (dinv) dinv[c] = pc ? ph.dinv[1] : ph.dinv[0];
+        if (rinv2) rinv2[c] = pc ? ph.wall[1] : ph.wall[0];
+        const float e = pc ? ph.eta[1] : ph.eta[0];
+        if (eta32) eta32[c] = e;
+        if (eta16) eta16[c] = __float2bfloat16_rn(e);
+        return;
     }
+    const double rc = rho_of(Fc, ra, rw);
+    if (!(rc > 0.0) || !isfinite(rc)) *bad = 1u;
+    const bool act = !ap.vol || ap.vol[c] > 0.0;
+    // the face to a neighbour: 0 if there is none; with cut cells scaled by its open fraction, and
+    // closed next to a cell with no fluid
+    auto face = [&](bool has, double Fn, int cn, const double* a, long long f) {
+        if (!has) return 0.0;
+        const int pn = phase_of(Fn);
+        double b;
+        if (pc < 2 && pn < 2) {
+            const int q = pc + pn;
+            b = q == 0 ? ph.face[0] : q == 1 ? ph.face[1] : ph.face[2];
+        } else {
+            b = 2.0 / __dadd_rn(rc, rho_of(Fn, ra, rw));
+        }
+        if (!a) return b;
+        return act && ap.vol[cn] > 0.0 ? __dmul_rn(a[f], b) : 0.0;
+    };
+    const long long fu = i + (long long)(d.nx + 1) * (j + (long long)d.ny * k);
+    const long long fv = i + (long long)d.nx * (j + (long long)(d.ny + 1) * k);
+    const long long up = c + (long long)d.sxy;
+    const double fx = face(hx0, Fx0, x0, ap.ax, fu);
+    const double fy = face(hy0, Fy0, c - d.nx, ap.ay, fv);
+    const double fz = face(hz0, Fz0, c - d.sxy, ap.az, c);
+    bx[c] = fx;
+    by[c] = fy;
+    bz[c] = fz;
     const double e = 0.5 * rc;
     if (eta32) eta32[c] = (float)e;
     if (eta16) eta16[c] = __float2bfloat16_rn((float)e);
-}
-
-// diag = bx[c] + by[c] + bz[c] + high faces (+ 2/rho_c on the top layer) (+ 2/rho_c for each
-// Dirichlet side/bottom wall the cell touches, x-, x+, y-, y+, z-), summed in that order;
-// top[i + nx j] = 2/rho_c of the top layer; rinv2[c] = 2/rho_c (only with Dirichlet walls).
-__global__ void k_setup_diag(Dims d, const double* __restrict__ F, double ra, double rw,
-                             const double* __restrict__ bx, const double* __restrict__ by,
-                             const double* __restrict__ bz, double* __restrict__ diag,
-                             double* __restrict__ dinv, double* __restrict__ top,
-                             double* __restrict__ rinv2, Apertures ap) {
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (tid >= d.n) return;
-    const int c = (int)tid;
-    const int i = c % d.nx, j = (c / d.nx) % d.ny, k = c / d.sxy;
-    const double t = 2.0 / rho_of(F[c], ra, rw);  // a boundary face's coefficient (unscaled)
-    if (k + 1 == d.nz && top) top[c - k * d.sxy] = t;
+    // a boundary face's coefficient, unscaled
+    double t = 0.0;
+    if (!hz1 || (d.walls & ~PERIODIC_X) || rinv2)
+        t = pc < 2 ? (pc ? ph.wall[1] : ph.wall[0]) : 2.0 / rc;
+    if (!hz1 && top) top[c - k * d.sxy] = t;
     if (rinv2) rinv2[c] = t;
-    if (ap.vol && !(ap.vol[c] > 0.0)) {
+    if (!act) {
         // cut cells: a cell with no fluid is inactive
         diag[c] = 1.0;
         if (dinv) dinv[c] = 1.0;
         return;
     }
-    const long long fu = i + (long long)(d.nx + 1) * (j + (long long)d.ny * k);
-    const long long fv = i + (long long)d.nx * (j + (long long)(d.ny + 1) * k);
     // a boundary term, scaled by its face's open fraction with cut cells
     auto bnd = [&](const double* a, long long f) { return a ? __dmul_rn(a[f], t) : t; };
-    double s = __dadd_rn(__dadd_rn(bx[c], by[c]), bz[c]);
-    if (i + 1 < d.nx) s = __dadd_rn(s, bx[c + 1]);
-    else if (d.walls & PERIODIC_X) s = __dadd_rn(s, bx[c + 1 - d.nx]);
-    if (j + 1 < d.ny) s = __dadd_rn(s, by[c + d.nx]);
-    if (k + 1 < d.nz) s = __dadd_rn(s, bz[c + d.sxy]);
-    else s = __dadd_rn(s, bnd(ap.az, c + (long long)d.sxy));
+    double s = __dadd_rn(__dadd_rn(fx, fy), fz);
+    // (the periodic wrap face is face 0 of the row)
+    if (hx1) s = __dadd_rn(s, face(true, Fx1, x1, ap.ax, i + 1 < d.nx ? fu + 1 : fu - i));
+    if (hy1) s = __dadd_rn(s, face(true, Fy1, c + d.nx, ap.ay, fv + d.nx));
+    s = __dadd_rn(s, hz1 ? face(true, Fz1, c + d.sxy, ap.az, up) : bnd(ap.az, up));
     if ((d.walls & 1) && i == 0) s = __dadd_rn(s, bnd(ap.ax, fu));
     if ((d.walls & 2) && i == d.nx - 1) s = __dadd_rn(s, bnd(ap.ax, fu + 1));
     if ((d.walls & 4) && j == 0) s = __dadd_rn(s, bnd(ap.ay, fv));
@@ -957,10 +1043,10 @@ void launch_setup(const Dims& d, const double* F, double ra, double rw, double* 
                   double* bz, double* diag, double* dinv, double* top, double* rinv2,
                   float* eta32, __nv_bfloat16* eta16, const Apertures& ap, unsigned* bad,
                   cudaStream_t st) {
-    k_setup_faces<<<blocks1d(d.n), 256, 0, st>>>(d, F, ra, rw, bx, by, bz, eta32, eta16, ap, bad);
-    k_setup_diag<<<blocks1d(d.n), 256, 0, st>>>(d, F, ra, rw, bx, by, bz, diag, dinv, top, rinv2,
-                                                ap);
-    counted(2);
+    k_setup<<<blocks1d(d.n), 256, 0, st>>>(d, FastDiv(d.nx), FastDiv(d.ny), F, ra, rw,
+                                           phases_of(ra, rw), bx, by, bz, diag, dinv, top, rinv2,
+                                           eta32, eta16, ap, bad);
+    counted(1);
 }
 
 void launch_scale(long long n, const double* s, double a, double* b, cudaStream_t st,

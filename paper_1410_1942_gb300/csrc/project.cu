@@ -32,8 +32,32 @@ constexpr int PT = 256;
 
 inline unsigned blocks_of(long long n) { return (unsigned)((n + PT - 1) / PT); }
 
+// Correctly rounded division by one divisor for all cells: with y = 1/h rounded to nearest,
+// q = a y, r = a - q h (exact by fused multiply-add) and q + r y rounded is the rounded quotient
+// (Markstein, "Computation of elementary functions on the IBM RISC System/6000", 1990; Brisebarre,
+// Muller and Raina, "Accelerating correctly rounded floating-point division when the divisor is
+// known in advance", 2004) as long as nothing under- or overflows: a's exponent is checked here
+// (zeros take q, which has the right sign), h's on the host.  Both passes are bound by the FP64
+// pipe, two operations a clock and SM, and the general division was most of their operations:
+// on 256x128x128 the projection took 286 us and takes 178, the divergence 100 and 66.
+struct DivBy {
+    double h, y;
+    int ok;
+    explicit DivBy(double h_) : h(h_), y(1.0 / h_) {
+        int e = 0;
+        std::frexp(h, &e);
+        ok = std::isfinite(h) && h > 0.0 && e > -100 && e < 100;
+    }
+    __device__ __forceinline__ double of(double a) const {
+        const unsigned ex = (unsigned)__double2hiint(a) & 0x7ff00000u;
+        const double q = __dmul_rn(a, y);
+        if (ok && ex - (123u << 20) < (1800u << 20)) return __fma_rn(__fma_rn(-q, h, a), y, q);
+        return ok && a == 0.0 ? q : __ddiv_rn(a, h);
+    }
+};
+
 // s_c = ((u_{i+1} - u_i) + (v_{j+1} - v_j) + (w_{k+1} - w_k)) / (h dt)
-__global__ void __launch_bounds__(PT) k_divergence(Dims d, double hd, const double* __restrict__ u,
+__global__ void __launch_bounds__(PT) k_divergence(Dims d, const __grid_constant__ DivBy hd, const double* __restrict__ u,
                                                    const double* __restrict__ v,
                                                    const double* __restrict__ w,
                                                    double* __restrict__ s, pcg::Apertures ap) {
@@ -54,22 +78,22 @@ __global__ void __launch_bounds__(PT) k_divergence(Dims d, double hd, const doub
         const double dv = __dsub_rn(__dmul_rn(ap.ay[fv + d.nx], v[fv + d.nx]),
                                     __dmul_rn(ap.ay[fv], v[fv]));
         const double dw = __dsub_rn(__dmul_rn(ap.az[up], w[up]), __dmul_rn(ap.az[c], w[c]));
-        s[c] = __ddiv_rn(__ddiv_rn(__dadd_rn(__dadd_rn(du, dv), dw), hd), ap.vol[c]);
+        s[c] = __ddiv_rn(hd.of(__dadd_rn(__dadd_rn(du, dv), dw)), ap.vol[c]);
         return;
     }
     const double du = __dsub_rn(u[fu + 1], u[fu]);
     const double dv = __dsub_rn(v[fv + d.nx], v[fv]);
     const double dw = __dsub_rn(w[c + (long long)d.sxy], w[c]);
-    s[c] = __ddiv_rn(__dadd_rn(__dadd_rn(du, dv), dw), hd);
+    s[c] = hd.of(__dadd_rn(__dadd_rn(du, dv), dw));
 }
 
 // q - dt (beta ((p_hi - p_lo) / h)), in that order
 __device__ __forceinline__ double corrected(double q, double dt, double beta, double p_hi,
-                                            double p_lo, double h) {
-    return __dsub_rn(q, __dmul_rn(dt, __dmul_rn(beta, __ddiv_rn(__dsub_rn(p_hi, p_lo), h))));
+                                            double p_lo, const DivBy& h) {
+    return __dsub_rn(q, __dmul_rn(dt, __dmul_rn(beta, h.of(__dsub_rn(p_hi, p_lo)))));
 }
 
-__global__ void __launch_bounds__(PT) k_project(Dims d, double h, double dt,
+__global__ void __launch_bounds__(PT) k_project(Dims d, const __grid_constant__ DivBy h, double dt,
                                                 const double* __restrict__ bx,
                                                 const double* __restrict__ by,
                                                 const double* __restrict__ bz,
@@ -231,7 +255,7 @@ extern "C" int poisson_divergence(poisson_t* H, const double* u, const double* v
         finish(H->st);
         return rc;
     }
-    k_divergence<<<blocks_of(d.n), PT, 0, H->st>>>(d, H->h * dt, U.dev, V.dev, W.dev, S.dev,
+    k_divergence<<<blocks_of(d.n), PT, 0, H->st>>>(d, DivBy(H->h * dt), U.dev, V.dev, W.dev, S.dev,
                                                   H->apertures());
     pcg::g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
     if (cudaGetLastError() != cudaSuccess) rc = POISSON_ECUDA;
@@ -256,7 +280,7 @@ extern "C" int poisson_project(poisson_t* H, double* u, double* v, double* w, co
         finish(H->st);
         return rc;
     }
-    k_project<<<blocks_of(d.n), PT, 0, H->st>>>(d, H->h, dt, H->bx, H->by, H->bz, H->top64,
+    k_project<<<blocks_of(d.n), PT, 0, H->st>>>(d, DivBy(H->h), dt, H->bx, H->by, H->bz, H->top64,
                                                 H->rinv2, P.dev, U.dev, V.dev, W.dev,
                                                 H->apertures());
     pcg::g_kernel_launches.fetch_add(1, std::memory_order_relaxed);
