@@ -36,8 +36,7 @@
 // m = i / 2 as well), so a warp's lanes, one per m, read neighbours at consecutive addresses: the
 // x neighbours of a cell of parity bit c (i = 2m + c) sit at m - 1 + c and m + c of the other
 // colour, its y and z neighbours at m.  Rings of 5 u' planes and 4 t planes; a segment of planes
-// [k0, k1) streams planes k0-2 .. k1+1 and runs two more steps without a new plane.  Tiles whose
-// cells and rings lie inside the grid in x and y take a stencil without boundary tests.  The
+// [k0, k1) streams planes k0-2 .. k1+1 and runs two more steps without a new plane.  The
 // faces are 1/(eta_c + eta_n) (eta = rho/2) formed on the fly as in the Jacobi kernels, so S is
 // the Schur complement of the same inner operator.  Work list, producer/consumer roles, bounded
 // waits, fixed-order float-float reductions and the finishing protocol are those of march1.cu.
@@ -89,24 +88,6 @@ struct LocalSolveRB {
 
 __device__ __forceinline__ float u_next_rb(float u, float s, float w, float al, float be) {
     return __fmaf_rn(-al, __fmaf_rn(be, s, w), u);
-}
-
-__device__ __forceinline__ int ring(int k, int n) { return (k + 4 * n) % n; }
-
-// The faces and diagonal of a cell whose x and y neighbours are all inside the grid (the
-// expressions of eta_stencil with its x and y tests dropped; the z tests are uniform per plane).
-__device__ __forceinline__ void eta_stencil_inner(const Dims& d, int k, float ec, float exm,
-                                                  float exp_, float eym, float eyp, float ezm,
-                                                  float ezp, Stencil<float>& w) {
-    w.xm = rcp_approx(ec + exm);
-    w.xp = rcp_approx(ec + exp_);
-    w.ym = rcp_approx(ec + eym);
-    w.yp = rcp_approx(ec + eyp);
-    w.zm = (k > 0) ? rcp_approx(ec + ezm) : ((d.walls & 16) ? rcp_approx(ec) : 0.f);
-    const bool top = (k + 1 == d.nz);
-    const float wzt = top ? rcp_approx(ec) : rcp_approx(ec + ezp);
-    w.zp = top ? 0.f : wzt;
-    w.D = w.xm + w.xp + w.ym + w.yp + w.zm + wzt;
 }
 
 template <int CX, int CY, int TYT, typename E, int NS>
@@ -178,7 +159,6 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
     const int lane = tx, warp = ty;
     auto stage = [&](int q) { return sm + (q % NS) * G::STAGE; };
     int np = 0;  // planes issued (producer lane 0)
-    int nc = 0;  // planes acquired (each consumer warp)
 
     // in: the buffer (0 or 1) of u, s^, w^ read by this sweep
     auto produce = [&](int in) {
@@ -213,181 +193,228 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
         }
     };
 
-    // step 1 on plane q: u' at compressed column jc (m = x0/2 - 2 + jc) of on-chip row r
-    auto step1 = [&](const unsigned char* S, float* Uq, float al, float be, int r, int jc) {
-        const int si = r * G::VW + G::VOFF - 2 + jc;
-        const float* Su = (const float*)(S + G::U);
-        const float* Ss = (const float*)(S + G::S);
-        const float* Sw = (const float*)(S + G::WV);
-        Uq[r * G::UC + jc] = u_next_rb(Su[si], Ss[si], Sw[si], al, be);
+    // What a thread's elements of the steps are is the same for every plane: worked out here once.
+    // (The index arithmetic, the rings' remainders and two forms of every stencil, with and without
+    // boundary tests, were half the kernel's instructions when each plane did them again: 59.3 us
+    // an iteration on 256x128x128 against 38.4, 204 and 138 on 512x256x128 with BF16 densities.)
+    // Steps 1 and 2 are spread over all consumer threads by flat element index (consecutive threads
+    // on consecutive columns); step 2 from the first thread and step 1 from the last, so the
+    // threads left with one t fewer take the extra u' values.
+    constexpr int N1 = (G::UPL + NC - 1) / NC, N2 = (G::TPL + NC - 1) / NC;
+    int si1[N1];  // step 1: byte offset in the halo boxes (the element's in a u' plane is e)
+    int ei2[N2], ui2[N2], rt2[N2], jt2[N2];  // step 2: offsets at parity 0 in eta and u', row, column
+#pragma unroll
+    for (int n = 0; n < N1; ++n) {
+        const int e = NC - 1 - tid + n * NC, r = e / G::UC;
+        si1[n] = (r * G::VW + G::VOFF - 2 + e - r * G::UC) * 4;
+    }
+#pragma unroll
+    for (int n = 0; n < N2; ++n) {
+        const int e = tid + n * NC, rt = e / G::TC, jt = e - rt * G::TC;
+        rt2[n] = rt;
+        jt2[n] = jt;
+        ei2[n] = (rt + 1) * G::EW + 2 * jt - 2 + G::EOFF;
+        ui2[n] = (rt + 1) * G::UC + jt;
+    }
+
+    // The six faces of the cell at eta position ei, from the planes below, of and above it.  Beyond a
+    // Neumann side rho/2 counts as infinite (face 0), beyond a Dirichlet side, the top included, as
+    // 0 (face 1/eta_c: what the boxes hold outside the grid, where u' and t are 0 too); edges: which
+    // of the sides x-, x+, y-, y+ are Neumann boundaries of this cell, floor0: its z- side is one.
+    auto faces = [&](const E* Em, const E* Ec, const E* Ep, int ei, int edges, bool floor0,
+                     Stencil<float>& w) {
+        const float inf = __int_as_float(0x7f800000);
+        const float ec = ld1(Ec + ei);
+        float xm = ld1(Ec + ei - 1), xp = ld1(Ec + ei + 1);
+        float ym = ld1(Ec + ei - G::EW), yp = ld1(Ec + ei + G::EW);
+        const float zm = floor0 ? inf : ld1(Em + ei), zp = ld1(Ep + ei);
+        if (edges & 1) xm = inf;
+        if (edges & 2) xp = inf;
+        if (edges & 4) ym = inf;
+        if (edges & 8) yp = inf;
+        w.xm = rcp_approx(ec + xm);
+        w.xp = rcp_approx(ec + xp);
+        w.ym = rcp_approx(ec + ym);
+        w.yp = rcp_approx(ec + yp);
+        w.zm = rcp_approx(ec + zm);
+        w.zp = rcp_approx(ec + zp);
+        w.D = w.xm + w.xp + w.ym + w.yp + w.zm + w.zp;
     };
 
-    // step 2 on plane kt: t of the red cell at compressed column jt (m = x0/2 - 1 + jt) of
-    // on-chip row rt (y = y0 - 1 + rt); 0 outside the grid
-    auto step2 = [&](const Dims& d, const Seg& sg, bool inner, int kt, const E* Em, const E* Ec,
-                     const E* Ep, const float* Um, const float* Uc, const float* Up, float* Tt,
-                     int rt, int jt) {
-        const int y = sg.y0 - 1 + rt;
-        const int pr = (y + kt) & 1;  // red: i + j + k even, i = 2m + pr
-        const int x = sg.x0 - 2 + 2 * jt + pr;
-        float t = 0.f;
-        if (inner || (x >= 0 && x < d.nx && y >= 0 && y < d.ny)) {
-            const int ei = (rt + 1) * G::EW + 2 * jt - 2 + pr + G::EOFF;
-            Stencil<float> w;
-            if (inner)
-                eta_stencil_inner(d, kt, ld1(Ec + ei), ld1(Ec + ei - 1), ld1(Ec + ei + 1),
-                                  ld1(Ec + ei - G::EW), ld1(Ec + ei + G::EW), ld1(Em + ei),
-                                  ld1(Ep + ei), w);
-            else
-                eta_stencil(d, x, y, kt, ld1(Ec + ei), ld1(Ec + ei - 1), ld1(Ec + ei + 1),
-                            ld1(Ec + ei - G::EW), ld1(Ec + ei + G::EW), ld1(Em + ei), ld1(Ep + ei),
-                            w);
-            const int ui = (rt + 1) * G::UC + jt;  // u' column of m - 1
-            float s = w.xm * Uc[ui + pr];
-            s += w.xp * Uc[ui + 1 + pr];
-            s += w.ym * Uc[ui + 1 - G::UC];
-            s += w.yp * Uc[ui + 1 + G::UC];
-            s += w.zm * Um[ui + 1];
-            s += w.zp * Up[ui + 1];
-            t = s * rcp_approx(w.D);
-        }
-        Tt[rt * G::TC + jt] = t;
-    };
-
+    int stc = 0, phc = 0;  // stage and phase of the next plane to acquire
     auto consume = [&](int in) {
         auto acquire = [&]() -> bool {
-            const int q = nc++;
+            const int st = stc, ph = phc;
+            if (++stc == NS) {
+                stc = 0;
+                phc ^= 1;
+            }
             if (s_fail) return false;
-            if (!mbar_wait_or(&full[q % NS], (q / NS) & 1, &s_fail)) {
+            if (!mbar_wait_or(&full[st], ph, &s_fail)) {
                 s_fail = 1;
                 return false;
             }
             return true;
         };
-        auto release = [&](int q) {
+        auto release = [&](int st) {
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[q % NS]);
+            if (lane == 0) mbar_arrive(&empty[st]);
         };
         const int out = in ^ 1;
         for (int ls = 0; ls < nseg; ++ls) {
             const Seg sg = s_seg[ls];
             const int l = sg.solve - first;
             if (!s_member[l]) continue;
-            const bool work = s_sol[l].done == RUNNING;
-            const Dims d = s_sol[l].d;
             const LocalSolveRB& Ls = s_sol[l];
+            const bool work = Ls.done == RUNNING;
+            const Dims d = Ls.d;
             const int nxh = d.nx >> 1;
             const float al = (float)Ls.alpha, be = (float)Ls.beta;
             const bool xs = !Ls.first;
             const int L = sg.k1 - sg.k0;
-            // the tile, its two rings of u' and the neighbours of its ring of t inside the grid
-            const bool inner = sg.x0 >= 4 && sg.x0 + G::W + 4 <= d.nx && sg.y0 >= 3 &&
-                               sg.y0 + G::HT + 3 <= d.ny;
-            const int p0 = nc;  // sequence number of plane k0 - 2
+            float *const gx = Ls.x, *const gp = Ls.p, *const gu = Ls.u[out], *const gs = Ls.s[out],
+                  *const gw = Ls.w[out];
+            const bool floorw = (d.walls & 16) != 0;  // the bottom is a Dirichlet wall
+            // Neumann sides of a cell in row y whose pair of columns is m: bits 0, 1 for the cell of
+            // parity 0, 1 (x- and x+), 2 and 3 for y- and y+; bit 4: inside the grid
+            auto sides = [&](int m, int y) {
+                int b = 0;
+                if (m == 0 && !(d.walls & 1)) b |= 1;
+                if (m == nxh - 1 && !(d.walls & 2)) b |= 2;
+                if (y == 0 && !(d.walls & 4)) b |= 4;
+                if (y == d.ny - 1 && !(d.walls & 8)) b |= 8;
+                if (m >= 0 && m < nxh && y >= 0 && y < d.ny) b |= 16;
+                return b;
+            };
+            int b2[N2], b3[CY], cb[CY];
+#pragma unroll
+            for (int n = 0; n < N2; ++n)
+                b2[n] = sides((sg.x0 >> 1) - 1 + jt2[n], sg.y0 - 1 + rt2[n]);
+            const int m = (sg.x0 >> 1) + lane;
+#pragma unroll
+            for (int n = 0; n < CY; ++n) {
+                const int y = sg.y0 + warp + n * TYT;
+                b3[n] = sides(m, y);
+                cb[n] = m + nxh * (y + d.ny * sg.k0);
+            }
+            const int plane = nxh * d.ny;
             float ag = 0.f, ad = 0.f, ar = 0.f;
+            // stages of planes q .. q - 5, rings of u' (q .. q - 4) and t (q - 2 .. q - 5)
+            int s0 = stc * G::STAGE, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0, rel = stc;
+            float *u0 = Ur, *u1 = Ur + 4 * G::UPL, *u2 = Ur + 3 * G::UPL, *u3 = Ur + 2 * G::UPL,
+                  *u4 = Ur + G::UPL;
+            float *t0 = Tr, *t1 = Tr + 3 * G::TPL, *t2 = Tr + 2 * G::TPL, *t3 = Tr + G::TPL;
             for (int off = 0; off < L + 6; ++off) {
-                const int q = sg.k0 - 2 + off, qs = p0 + off;
+                const int q = sg.k0 - 2 + off;
                 const bool arrives = off < L + 4;
                 const bool ok = arrives ? acquire() : !s_fail;
                 if (ok && work) {
-                    // Steps 1 and 2 are spread over all consumer threads by flat element index
-                    // (consecutive threads on consecutive columns); step 2 from the first thread
-                    // and step 1 from the last, so the threads left with one t fewer take the
-                    // extra u' values.
                     if (arrives) {
                         // step 1: u' of plane q on the tile and two rings
-                        const unsigned char* S = stage(qs);
-                        float* Uq = Ur + ring(q, G::RINGU) * G::UPL;
-                        for (int e = NC - 1 - tid; e < G::UPL; e += NC) {
-                            const int r = e / G::UC;
-                            step1(S, Uq, al, be, r, e - r * G::UC);
+                        const unsigned char* const S = sm + s0;
+#pragma unroll
+                        for (int n = 0; n < N1; ++n) {
+                            const int e = NC - 1 - tid + n * NC;
+                            if ((n + 1) * NC <= G::UPL || e < G::UPL)
+                                u0[e] = u_next_rb(*(const float*)(S + G::U + si1[n]),
+                                                  *(const float*)(S + G::S + si1[n]),
+                                                  *(const float*)(S + G::WV + si1[n]), al, be);
                         }
                     }
                     const int kt = q - 2;
                     if (off >= 3 && off <= L + 4) {
-                        // step 2: t of plane kt = q - 2 on the red cells of the tile and one ring
-                        float* Tt = Tr + ring(kt, G::RINGT) * G::TPL;
-                        if (kt < 0 || kt >= d.nz) {
-                            for (int e = tid; e < G::TPL; e += NC) Tt[e] = 0.f;
-                        } else {
-                            const float* Um = Ur + ring(kt - 1, G::RINGU) * G::UPL;
-                            const float* Uc = Ur + ring(kt, G::RINGU) * G::UPL;
-                            const float* Up = Ur + ring(kt + 1, G::RINGU) * G::UPL;
-                            const E* Em = (const E*)(stage(qs - 3) + G::ETA);
-                            const E* Ec = (const E*)(stage(qs - 2) + G::ETA);
-                            const E* Ep = (const E*)(stage(qs - 1) + G::ETA);
-                            for (int e = tid; e < G::TPL; e += NC) {
-                                const int rt = e / G::TC;
-                                step2(d, sg, inner, kt, Em, Ec, Ep, Um, Uc, Up, Tt, rt,
-                                      e - rt * G::TC);
+                        // step 2: t of plane kt on the red cells (i + j + k even, i = 2m + pr) of
+                        // the tile and one ring; 0 outside the grid
+                        const E* const Em = (const E*)(sm + s3 + G::ETA);
+                        const E* const Ec = (const E*)(sm + s2 + G::ETA);
+                        const E* const Ep = (const E*)(sm + s1 + G::ETA);
+                        const bool inside = kt >= 0 && kt < d.nz, floor0 = kt == 0 && !floorw;
+#pragma unroll
+                        for (int n = 0; n < N2; ++n) {
+                            const int e = tid + n * NC;
+                            if ((n + 1) * NC > G::TPL && e >= G::TPL) continue;
+                            float t = 0.f;
+                            if (inside) {
+                                const int pr = (rt2[n] + 1 + kt) & 1, b = b2[n];
+                                const int edges = (b & 12) | (b & (1 << pr));
+                                Stencil<float> w;
+                                faces(Em, Ec, Ep, ei2[n] + pr, edges, floor0, w);
+                                const int ui = ui2[n];  // u' column of m - 1
+                                float v = w.xm * u2[ui + pr];
+                                v += w.xp * u2[ui + 1 + pr];
+                                v += w.ym * u2[ui + 1 - G::UC];
+                                v += w.yp * u2[ui + 1 + G::UC];
+                                v += w.zm * u3[ui + 1];
+                                v += w.zp * u1[ui + 1];
+                                t = (b & 16) ? v * rcp_approx(w.D) : 0.f;
                             }
+                            t0[e] = t;
                         }
                     }
                     const int k = q - 4;
                     if (off >= 6) {
-                        // step 3: S u' of plane k = q - 4 on the tile's black cells and updates
-                        const unsigned char* S = stage(qs - 4);
-                        const float* Su = (const float*)(S + G::U);
-                        const float* Ss = (const float*)(S + G::S);
-                        const float* Sw = (const float*)(S + G::WV);
-                        const float* Sx = (const float*)(S + G::X);
-                        const float* Sp = (const float*)(S + G::P);
-                        const E* Em = (const E*)(stage(qs - 5) + G::ETA);
-                        const E* Ec = (const E*)(S + G::ETA);
-                        const E* Ep = (const E*)(stage(qs - 3) + G::ETA);
-                        const float* Tm = Tr + ring(k - 1, G::RINGT) * G::TPL;
-                        const float* Tc = Tr + ring(k, G::RINGT) * G::TPL;
-                        const float* Tp = Tr + ring(k + 1, G::RINGT) * G::TPL;
-                        const float* Uc = Ur + ring(k, G::RINGU) * G::UPL;
-                        const int m = sg.x0 / 2 + lane;
-                        for (int r = warp; r < G::HT; r += TYT) {
-                            const int y = sg.y0 + r;
-                            if (!inner && (y >= d.ny || m >= nxh)) continue;
-                            const int pb = (y + k + 1) & 1;  // black: i = 2m + pb
-                            const int ei = (r + 2) * G::EW + 2 * lane + pb + G::EOFF;
-                            Stencil<float> w;
-                            if (inner)
-                                eta_stencil_inner(d, k, ld1(Ec + ei), ld1(Ec + ei - 1),
-                                                  ld1(Ec + ei + 1), ld1(Ec + ei - G::EW),
-                                                  ld1(Ec + ei + G::EW), ld1(Em + ei),
-                                                  ld1(Ep + ei), w);
-                            else
-                                eta_stencil(d, sg.x0 + 2 * lane + pb, y, k, ld1(Ec + ei),
-                                            ld1(Ec + ei - 1), ld1(Ec + ei + 1),
-                                            ld1(Ec + ei - G::EW), ld1(Ec + ei + G::EW),
-                                            ld1(Em + ei), ld1(Ep + ei), w);
-                            const int ti = (r + 1) * G::TC + lane;  // t column of m - 1
-                            float s = w.xm * Tc[ti + pb];
-                            s += w.xp * Tc[ti + 1 + pb];
-                            s += w.ym * Tc[ti + 1 - G::TC];
-                            s += w.yp * Tc[ti + 1 + G::TC];
-                            s += w.zm * Tm[ti + 1];
-                            s += w.zp * Tp[ti + 1];
-                            const float ub = Uc[(r + 2) * G::UC + lane + 2];
-                            const float su = w.D * ub - s;
-                            const int si = (r + 2) * G::VW + G::VOFF + lane;
-                            const float pn = __fmaf_rn(be, Sp[r * G::WB + lane], Su[si]);
-                            const float sn = __fmaf_rn(be, Ss[si], Sw[si]);
-                            const float wn = su * rcp_approx(w.D);
-                            const size_t cb = (size_t)m + (size_t)nxh * (y + (size_t)d.ny * k);
-                            if (xs) Ls.x[cb] = __fmaf_rn(al, pn, Sx[r * G::WB + lane]);
-                            Ls.p[cb] = pn;
-                            Ls.u[out][cb] = ub;
-                            Ls.s[out][cb] = sn;
-                            Ls.w[out][cb] = wn;
-                            const float du = w.D * ub;
-                            ag += du * ub;
-                            ad += su * ub;
-                            ar += du * du;
+                        // step 3: S u' of plane k on the tile's black cells (i = 2m + pb) and updates
+                        const unsigned char* const S = sm + s4;
+                        const float* const Su = (const float*)(S + G::U);
+                        const float* const Ss = (const float*)(S + G::S);
+                        const float* const Sw = (const float*)(S + G::WV);
+                        const float* const Sx = (const float*)(S + G::X);
+                        const float* const Sp = (const float*)(S + G::P);
+                        const E* const Em = (const E*)(sm + s5 + G::ETA);
+                        const E* const Ec = (const E*)(S + G::ETA);
+                        const E* const Ep = (const E*)(sm + s3 + G::ETA);
+                        const bool floor0 = k == 0 && !floorw;
+#pragma unroll
+                        for (int n = 0; n < CY; ++n) {
+                            const int r = warp + n * TYT, b = b3[n];
+                            if (b & 16) {
+                                const int pb = (r + k + 1) & 1;
+                                Stencil<float> w;
+                                faces(Em, Ec, Ep, (r + 2) * G::EW + 2 * lane + pb + G::EOFF,
+                                      (b & 12) | (b & (1 << pb)), floor0, w);
+                                const int ti = (r + 1) * G::TC + lane;  // t column of m - 1
+                                float v = w.xm * t2[ti + pb];
+                                v += w.xp * t2[ti + 1 + pb];
+                                v += w.ym * t2[ti + 1 - G::TC];
+                                v += w.yp * t2[ti + 1 + G::TC];
+                                v += w.zm * t3[ti + 1];
+                                v += w.zp * t1[ti + 1];
+                                const float ub = u4[(r + 2) * G::UC + lane + 2];
+                                const float du = w.D * ub, su = du - v;
+                                const int si = (r + 2) * G::VW + G::VOFF + lane;
+                                const float pn = __fmaf_rn(be, Sp[r * G::WB + lane], Su[si]);
+                                const float sn = __fmaf_rn(be, Ss[si], Sw[si]);
+                                const float wn = su * rcp_approx(w.D);
+                                const int c = cb[n];
+                                if (xs) gx[c] = __fmaf_rn(al, pn, Sx[r * G::WB + lane]);
+                                gp[c] = pn;
+                                gu[c] = ub;
+                                gs[c] = sn;
+                                gw[c] = wn;
+                                ag += du * ub;
+                                ad += su * ub;
+                                ar += du * du;
+                            }
+                            cb[n] += plane;
                         }
                     }
                 }
                 named_sync(1, NC);
-                if (off >= 5) release(qs - 5);
+                if (off >= 5) {
+                    release(rel);
+                    rel = rel + 1 == NS ? 0 : rel + 1;
+                }
+                s5 = s4, s4 = s3, s3 = s2, s2 = s1, s1 = s0;
+                s0 = s0 + G::STAGE == NS * G::STAGE ? 0 : s0 + G::STAGE;
+                float* const tu = u4;
+                u4 = u3, u3 = u2, u2 = u1, u1 = u0, u0 = tu;
+                float* const tt = t3;
+                t3 = t2, t2 = t1, t1 = t0, t0 = tt;
             }
-            release(p0 + L + 1);
-            release(p0 + L + 2);
-            release(p0 + L + 3);
+            for (int n = 0; n < 3; ++n) {
+                release(rel);
+                rel = rel + 1 == NS ? 0 : rel + 1;
+            }
             // the segment's partial sums (gamma, delta, rho), over the consumer warps
             const float v[3] = {ag, ad, ar};
             segment_partials<3>(v, a.part_b + 3 * (size_t)s_seg[ls].slot, reinterpret_cast<ff*>(red),
