@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
     // What a thread's elements of the steps are is the same for every plane: worked out here once.
     // (The index arithmetic, the rings' remainders and two forms of every stencil, with and without
     // boundary tests, were half the kernel's instructions when each plane did them again: 59.3 us
-    // an iteration on 256x128x128 against 38.4, 204 and 138 on 512x256x128 with BF16 densities.)
+    // an iteration on 256x128x128 against 37.2, 204 and 135 on 512x256x128 with BF16 densities.)
     // Steps 1 and 2 are spread over all consumer threads by flat element index (consecutive threads
     // on consecutive columns); step 2 from the first thread and step 1 from the last, so the
     // threads left with one t fewer take the extra u' values.
@@ -210,7 +210,8 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
     }
 #pragma unroll
     for (int n = 0; n < N2; ++n) {
-        const int e = tid + n * NC, rt = e / G::TC, jt = e - rt * G::TC;
+        // (a thread without an n-th element computes the last one again and stores nothing)
+        const int e = min(tid + n * NC, G::TPL - 1), rt = e / G::TC, jt = e - rt * G::TC;
         rt2[n] = rt;
         jt2[n] = jt;
         ei2[n] = (rt + 1) * G::EW + 2 * jt - 2 + G::EOFF;
@@ -329,16 +330,14 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
                         const E* const Ec = (const E*)(sm + s2 + G::ETA);
                         const E* const Ep = (const E*)(sm + s1 + G::ETA);
                         const bool inside = kt >= 0 && kt < d.nz, floor0 = kt == 0 && !floorw;
+                        if (inside) {
+                            // (every element in one straight line, stores last: their loads overlap)
+                            float t[N2];
 #pragma unroll
-                        for (int n = 0; n < N2; ++n) {
-                            const int e = tid + n * NC;
-                            if ((n + 1) * NC > G::TPL && e >= G::TPL) continue;
-                            float t = 0.f;
-                            if (inside) {
+                            for (int n = 0; n < N2; ++n) {
                                 const int pr = (rt2[n] + 1 + kt) & 1, b = b2[n];
-                                const int edges = (b & 12) | (b & (1 << pr));
                                 Stencil<float> w;
-                                faces(Em, Ec, Ep, ei2[n] + pr, edges, floor0, w);
+                                faces(Em, Ec, Ep, ei2[n] + pr, (b & 12) | (b & (1 << pr)), floor0, w);
                                 const int ui = ui2[n];  // u' column of m - 1
                                 float v = w.xm * u2[ui + pr];
                                 v += w.xp * u2[ui + 1 + pr];
@@ -346,9 +345,14 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
                                 v += w.yp * u2[ui + 1 + G::UC];
                                 v += w.zm * u3[ui + 1];
                                 v += w.zp * u1[ui + 1];
-                                t = (b & 16) ? v * rcp_approx(w.D) : 0.f;
+                                t[n] = (b & 16) ? v * rcp_approx(w.D) : 0.f;
                             }
-                            t0[e] = t;
+#pragma unroll
+                            for (int n = 0; n < N2; ++n)
+                                if ((n + 1) * NC <= G::TPL || tid + n * NC < G::TPL)
+                                    t0[tid + n * NC] = t[n];
+                        } else {
+                            for (int e = tid; e < G::TPL; e += NC) t0[e] = 0.f;
                         }
                     }
                     const int k = q - 4;
@@ -364,36 +368,41 @@ __global__ void __launch_bounds__(32 * (TYT + 1), 2) k_rb_ws(PcgArgs a) {
                         const E* const Ec = (const E*)(S + G::ETA);
                         const E* const Ep = (const E*)(sm + s3 + G::ETA);
                         const bool floor0 = k == 0 && !floorw;
+                        float pn[CY], sn[CY], wn[CY], ub[CY], xn[CY];
 #pragma unroll
                         for (int n = 0; n < CY; ++n) {
-                            const int r = warp + n * TYT, b = b3[n];
-                            if (b & 16) {
-                                const int pb = (r + k + 1) & 1;
-                                Stencil<float> w;
-                                faces(Em, Ec, Ep, (r + 2) * G::EW + 2 * lane + pb + G::EOFF,
-                                      (b & 12) | (b & (1 << pb)), floor0, w);
-                                const int ti = (r + 1) * G::TC + lane;  // t column of m - 1
-                                float v = w.xm * t2[ti + pb];
-                                v += w.xp * t2[ti + 1 + pb];
-                                v += w.ym * t2[ti + 1 - G::TC];
-                                v += w.yp * t2[ti + 1 + G::TC];
-                                v += w.zm * t3[ti + 1];
-                                v += w.zp * t1[ti + 1];
-                                const float ub = u4[(r + 2) * G::UC + lane + 2];
-                                const float du = w.D * ub, su = du - v;
-                                const int si = (r + 2) * G::VW + G::VOFF + lane;
-                                const float pn = __fmaf_rn(be, Sp[r * G::WB + lane], Su[si]);
-                                const float sn = __fmaf_rn(be, Ss[si], Sw[si]);
-                                const float wn = su * rcp_approx(w.D);
-                                const int c = cb[n];
-                                if (xs) gx[c] = __fmaf_rn(al, pn, Sx[r * G::WB + lane]);
-                                gp[c] = pn;
-                                gu[c] = ub;
-                                gs[c] = sn;
-                                gw[c] = wn;
-                                ag += du * ub;
-                                ad += su * ub;
-                                ar += du * du;
+                            const int r = warp + n * TYT, b = b3[n], pb = (r + k + 1) & 1;
+                            Stencil<float> w;
+                            faces(Em, Ec, Ep, (r + 2) * G::EW + 2 * lane + pb + G::EOFF,
+                                  (b & 12) | (b & (1 << pb)), floor0, w);
+                            const int ti = (r + 1) * G::TC + lane;  // t column of m - 1
+                            float v = w.xm * t2[ti + pb];
+                            v += w.xp * t2[ti + 1 + pb];
+                            v += w.ym * t2[ti + 1 - G::TC];
+                            v += w.yp * t2[ti + 1 + G::TC];
+                            v += w.zm * t3[ti + 1];
+                            v += w.zp * t1[ti + 1];
+                            ub[n] = u4[(r + 2) * G::UC + lane + 2];
+                            const float du = w.D * ub[n], su = du - v;
+                            const int si = (r + 2) * G::VW + G::VOFF + lane, ci = r * G::WB + lane;
+                            pn[n] = __fmaf_rn(be, Sp[ci], Su[si]);
+                            sn[n] = __fmaf_rn(be, Ss[si], Sw[si]);
+                            wn[n] = su * rcp_approx(w.D);
+                            xn[n] = xs ? __fmaf_rn(al, pn[n], Sx[ci]) : 0.f;
+                            const bool cell = (b & 16) != 0;
+                            ag += cell ? du * ub[n] : 0.f;
+                            ad += cell ? su * ub[n] : 0.f;
+                            ar += cell ? du * du : 0.f;
+                        }
+#pragma unroll
+                        for (int n = 0; n < CY; ++n) {
+                            const int c = cb[n];
+                            if (b3[n] & 16) {
+                                if (xs) gx[c] = xn[n];
+                                gp[c] = pn[n];
+                                gu[c] = ub[n];
+                                gs[c] = sn[n];
+                                gw[c] = wn[n];
                             }
                             cb[n] += plane;
                         }
