@@ -82,7 +82,7 @@ __device__ __forceinline__ bool x_sweep(const LocalSolve1& L) { return !L.first 
 // ROWS_ANY, rows of any length stored at a pitch of whole 32 bytes (the tensor maps end at nx, so
 // what lies beyond reads as zero; the last thread of an odd row owns one column).  Separate
 // instantiations, so that the plain kernel carries none of it.  A 250 x 125 x 90 grid, which the
-// column kernels took 77 us an iteration for, takes 23 (301 x 151 x 120: 130 and 43).
+// column kernels took 77 us an iteration for, takes 22 (301 x 151 x 120: 130 and 43).
 template <int CX, int CY, int TYT, typename E, int NS, int MODE>
 __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1_ws(PcgArgs a) {
     using G = Geo1<CX, CY, TYT, E>;
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
 
     const int r0 = 1 + CY * ty, cv = G::VOFF + CX * tx, ce = G::EOFF + CX * tx, cc = CX * tx;
     const int warp = ty, lane = tx;
-    auto stage = [&](int q) { return sm + (q % NS) * G::STAGE; };
+    auto stage = [&](int q) { return sm + ((unsigned)q % NS) * G::STAGE; };
     int np = 0;  // planes issued (producer lane 0)
     int nc = 0;  // planes acquired (each consumer warp)
 
@@ -250,7 +250,14 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                         wzl[y][x] = (sg.k0 > 0 || (d.walls & 16)) ? rcp_approx(ec[y][x] + em[y][x]) : 0.f;
             }
             float ag = 0.f, ad = 0.f, ar = 0.f;
-            for (int k = sg.k0; k < sg.k1; ++k) {
+            // the thread's arrays and its cell of the plane: read from the record again after every
+            // store, which may alias it, they made an iteration 30.2 us on 256x128x128 (29.9 now),
+            // 119.7 on 512x256x128 with BF16 densities (116.4) and 22.8 on 250x125x90 (21.7)
+            const int rp = MODE != ROWS_PLAIN ? s_sol[l].nxp : d.nx;  // u, s^ and w^'s row
+            size_t cell = (size_t)i0 + (size_t)(PER ? d.nx : rp) * (j0 + (size_t)d.ny * sg.k0);
+            float *const gx = s_sol[l].x, *const gp = s_sol[l].p, *const gu = s_sol[l].u[out],
+                  *const gs = s_sol[l].s[out], *const gw = s_sol[l].w[out];
+            for (int k = sg.k0; k < sg.k1; ++k, cell += (size_t)(PER ? d.nx : rp) * d.ny) {
                 const int qc = p0 + 1 + (k - sg.k0), qn = qc + 1;
                 ok = acquire();  // plane k+1
                 if (ok && work) {
@@ -307,25 +314,21 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                                     ad += in ? qv[y][x] * uc[y][x] : 0.f;
                                     ar += du * du;
                                 }
-                                const size_t c =
-                                    (size_t)i0 + (size_t)(RAG ? s_sol[l].nxp : d.nx) *
-                                                     (j0 + y + (size_t)d.ny * k);
-                                if (xs) st_row<CX>(s_sol[l].x + c, xn);
-                                st_row<CX>(s_sol[l].p + c, pn);
-                                const LocalSolve1& Ls = s_sol[l];
-                                const size_t row = (size_t)(MODE != ROWS_PLAIN ? Ls.nxp : d.nx) *
-                                                   (j0 + y + (size_t)d.ny * k);
-                                const size_t cp = row + i0 + (PER ? PAD_V : 0);
-                                st_row<CX>(Ls.u[out] + cp, uc[y]);
-                                st_row<CX>(Ls.s[out] + cp, sn);
-                                st_row<CX>(Ls.w[out] + cp, wn);
+                                const size_t c = cell + (size_t)(PER ? d.nx : rp) * y;
+                                if (xs) st_row<CX>(gx + c, xn);
+                                st_row<CX>(gp + c, pn);
+                                const size_t row = PER ? (size_t)rp * (j0 + y + (size_t)d.ny * k) : 0;
+                                const size_t cp = PER ? row + i0 + PAD_V : c;
+                                st_row<CX>(gu + cp, uc[y]);
+                                st_row<CX>(gs + cp, sn);
+                                st_row<CX>(gw + cp, wn);
                                 if (PER && (i0 < PAD_V || i0 >= d.nx - PAD_V)) {
                                     // the ghost copy at the other end of the padded row
                                     const long long cg = (long long)row + i0 + PAD_V +
                                                          (i0 < PAD_V ? d.nx : -d.nx);
-                                    st_row<CX>(Ls.u[out] + cg, uc[y]);
-                                    st_row<CX>(Ls.s[out] + cg, sn);
-                                    st_row<CX>(Ls.w[out] + cg, wn);
+                                    st_row<CX>(gu + cg, uc[y]);
+                                    st_row<CX>(gs + cg, sn);
+                                    st_row<CX>(gw + cg, wn);
                                 }
                             }
                         }
