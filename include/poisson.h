@@ -352,6 +352,11 @@ int poisson_residual_noalloc(int nx, int ny, int nz, double h, const double* F, 
  * persistent launch: POISSON_FP64, RBSSOR, MG, cut cells, nx % 8 != 0, tile = -1). */
 int poisson_test_unreachable_barrier(poisson_t* h, int extra);
 
+/* The same for a handle whose PCG runs on chip, of any precision and with cut cells: with extra = 1
+ * its sweeps wait for the sums of one box more than the solve has (deadline 1 s).  It concerns
+ * poisson_solve, not batches.  Errors: EINVAL (NULL, extra not 0 or 1, not an on-chip handle). */
+int poisson_test_unreachable_box(poisson_t* h, int extra);
+
 /* Testing aids for the allocation error paths (the failure is injected on the host; nothing
  * faults on the GPU).  poisson_test_fail_alloc(n): the n-th device or pinned-host allocation the
  * library makes from now on, in any thread, fails as if memory were exhausted, and the call that

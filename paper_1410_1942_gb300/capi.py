@@ -34,7 +34,7 @@ EXPORTS = ["poisson_default_opts", "poisson_create", "poisson_destroy", "poisson
            "poisson_divergence", "poisson_project", "poisson_set_apertures", "poisson_strerror",
            "poisson_version", "poisson_test_unreachable_barrier", "poisson_hydrostatic_force",
            "poisson_required_bytes", "poisson_handle_bytes", "poisson_test_fail_alloc",
-           "poisson_test_live_allocations"]
+           "poisson_test_live_allocations", "poisson_test_unreachable_box"]
 K_CG_A, K_CG_B, K_RESIDUAL, K_OTHER, K_PCG = 0, 1, 2, 3, 4
 K_NAMES = ["cg_phase_a", "cg_phase_b", "residual64", "other", "pcg_persistent"]
 
@@ -123,6 +123,8 @@ def load(path=None):
     lib.poisson_hydrostatic_force.restype = i
     lib.poisson_test_unreachable_barrier.argtypes = [vp, i]
     lib.poisson_test_unreachable_barrier.restype = i
+    lib.poisson_test_unreachable_box.argtypes = [vp, i]
+    lib.poisson_test_unreachable_box.restype = i
     lib.poisson_test_fail_alloc.argtypes = [i]
     lib.poisson_test_fail_alloc.restype = i
     lib.poisson_test_live_allocations.argtypes = [ctypes.POINTER(ctypes.c_longlong)]
@@ -261,6 +263,11 @@ class Poisson:
         CTAs more than they launch (0 restores), so a solve ends with ETIMEOUT."""
         _check(load().poisson_test_unreachable_barrier(self._h, int(extra)),
                "poisson_test_unreachable_barrier")
+
+    def test_unreachable_box(self, extra):
+        """Testing aid: the on-chip PCG's sweeps wait for one box more than there are (0 restores)."""
+        _check(load().poisson_test_unreachable_box(self._h, int(extra)),
+               "poisson_test_unreachable_box")
 
     def device_bytes(self):
         """Device bytes the handle holds (poisson_handle_bytes)."""

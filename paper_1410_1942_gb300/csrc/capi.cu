@@ -1214,6 +1214,12 @@ extern "C" int poisson_test_unreachable_barrier(poisson_t* H, int extra) {
     return POISSON_OK;
 }
 
+extern "C" int poisson_test_unreachable_box(poisson_t* H, int extra) {
+    if (!H || extra < 0 || extra > 1 || !H->res) return POISSON_EINVAL;
+    H->rplan.extra = extra;
+    return POISSON_OK;
+}
+
 extern "C" int poisson_solve(poisson_t* H, const double* rhs, double* p, double tol,
                              poisson_stats* stats) {
     if (!H || !rhs || !p || !(tol > 0.0)) return POISSON_EINVAL;

@@ -282,9 +282,16 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
     __shared__ T tot[RANKS / 32][3];
     __shared__ double s_dec[2];
     __shared__ int s_state, s_iter;
-    __shared__ volatile int s_fail;
+    // A wait that ran out: for a sum, written before the decision's barrier and read after it; for a
+    // halo word, written after that barrier and read after the sweep's last one.  One flag for
+    // both could be set by a late halo poll while slower warps still read it after the decision,
+    // and part of the CTA would leave while the rest waits at a barrier.
+    __shared__ volatile int s_fail, s_late;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_fail = 0;
+    if (tid == 0) {
+        s_fail = 0;
+        s_late = 0;
+    }
     for (int it = a.cta_task[blockIdx.x]; it < a.cta_task[blockIdx.x + 1]; ++it) {
         const ResTask& tk = a.tasks[it];
         const ResSolve& sv = a.solves[tk.solve];
@@ -700,7 +707,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
             if (late) {
                 Deadline dl;
                 while ((late = get_halo(late)) != 0)
-                    if (!dl.more(a.error)) { s_fail = 1; break; }
+                    if (!dl.more(a.error)) { s_late = 1; break; }
             }
 #pragma unroll
             for (int q = 0; q < HQ; ++q) {
@@ -710,7 +717,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
                 }
             }
             __syncthreads();
-            if (s_fail) { state = TIMEDOUT; break; }
+            if (s_late) { state = TIMEDOUT; break; }
         }
         // the correction and the scalars
         V* const xg = reinterpret_cast<V*>(sv.x);

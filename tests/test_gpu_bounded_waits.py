@@ -1,0 +1,56 @@
+"""The bounded waits of the on-chip PCG and of the V-cycle's fine passes: a wait that runs out ends the
+solve with ETIMEOUT (nothing faults or hangs), and the same handle then solves as if nothing had
+happened."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1410_1942_gb300 import build, capi, inputs
+
+pytestmark = pytest.mark.gpu
+
+L2_TOL = 1e-6
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    assert torch.cuda.is_available()
+    build.build()
+    capi.load()
+
+
+def _check(op, b, p, tol):
+    rel = oracle.rel_residual(op, b, p)
+    assert rel <= tol * (1 + 1e-6), rel
+    ref = oracle.pcg(op, b, tol=1e-12, precond="ssor").x
+    assert np.linalg.norm(p - ref) <= L2_TOL * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("prec,cut", [("fp64", False), ("fp64", True), ("fp32", True),
+                                      ("bf16", False)])
+def test_an_unreachable_box_times_out_in_every_precision(prec, cut):
+    c = inputs.strut_case(64, 32, 32, seed=2)
+    g = c.grid
+    aps = None
+    if cut:
+        Lx, Ly, _ = g.lengths
+        aps = inputs.cut_apertures(
+            g, lambda x, y, z: inputs.ellipse_sdf(x, y, 0.5 * Lx, 0.5 * Ly, 0.3 * Lx, 0.2 * Ly))
+    with capi.Poisson(g.nx, g.ny, g.nz, g.h, precision=prec) as s:
+        if cut:
+            s.set_apertures(*aps)
+        s.set_density(c.F)
+        assert "on chip" in s.describe(), s.describe()
+        s.test_unreachable_box(1)
+        p = np.zeros(g.shape)
+        rc, _ = s.solve(c.s, p, c.tol, allow=(capi.ETIMEOUT,))
+        assert rc == capi.ETIMEOUT and np.all(np.isfinite(p))
+        s.test_unreachable_box(0)
+        p = np.zeros(g.shape)
+        rc, _ = s.solve(c.s, p, c.tol)
+        assert rc == capi.OK
+    if cut:
+        _check(oracle.operator(c.F, apertures=aps), oracle.rhs(c.s, g.h, aps[3]), p, c.tol)
+    else:
+        _check(oracle.operator(c.F), oracle.rhs(c.s, g.h), p, c.tol)
