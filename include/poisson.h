@@ -357,6 +357,11 @@ int poisson_test_unreachable_barrier(poisson_t* h, int extra);
  * poisson_solve, not batches.  Errors: EINVAL (NULL, extra not 0 or 1, not an on-chip handle). */
 int poisson_test_unreachable_box(poisson_t* h, int extra);
 
+/* The limit, in seconds (default and most: 1), after which a wait of an on-chip PCG gives up when
+ * no solve of its launch has made progress meanwhile; in batches too.
+ * Errors: EINVAL (NULL, seconds not in (0, 1], not an on-chip handle). */
+int poisson_test_wait_limit(poisson_t* h, double seconds);
+
 /* Testing aids for the allocation error paths (the failure is injected on the host; nothing
  * faults on the GPU).  poisson_test_fail_alloc(n): the n-th device or pinned-host allocation the
  * library makes from now on, in any thread, fails as if memory were exhausted, and the call that

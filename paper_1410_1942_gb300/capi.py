@@ -34,7 +34,8 @@ EXPORTS = ["poisson_default_opts", "poisson_create", "poisson_destroy", "poisson
            "poisson_divergence", "poisson_project", "poisson_set_apertures", "poisson_strerror",
            "poisson_version", "poisson_test_unreachable_barrier", "poisson_hydrostatic_force",
            "poisson_required_bytes", "poisson_handle_bytes", "poisson_test_fail_alloc",
-           "poisson_test_live_allocations", "poisson_test_unreachable_box"]
+           "poisson_test_live_allocations", "poisson_test_unreachable_box",
+           "poisson_test_wait_limit"]
 K_CG_A, K_CG_B, K_RESIDUAL, K_OTHER, K_PCG = 0, 1, 2, 3, 4
 K_NAMES = ["cg_phase_a", "cg_phase_b", "residual64", "other", "pcg_persistent"]
 
@@ -125,6 +126,8 @@ def load(path=None):
     lib.poisson_test_unreachable_barrier.restype = i
     lib.poisson_test_unreachable_box.argtypes = [vp, i]
     lib.poisson_test_unreachable_box.restype = i
+    lib.poisson_test_wait_limit.argtypes = [vp, d]
+    lib.poisson_test_wait_limit.restype = i
     lib.poisson_test_fail_alloc.argtypes = [i]
     lib.poisson_test_fail_alloc.restype = i
     lib.poisson_test_live_allocations.argtypes = [ctypes.POINTER(ctypes.c_longlong)]
@@ -268,6 +271,10 @@ class Poisson:
         """Testing aid: the on-chip PCG's sweeps wait for one box more than there are (0 restores)."""
         _check(load().poisson_test_unreachable_box(self._h, int(extra)),
                "poisson_test_unreachable_box")
+
+    def test_wait_limit(self, seconds):
+        """Testing aid: how long the on-chip PCG's waits may see no progress (1 s by default)."""
+        _check(load().poisson_test_wait_limit(self._h, float(seconds)), "poisson_test_wait_limit")
 
     def device_bytes(self):
         """Device bytes the handle holds (poisson_handle_bytes)."""

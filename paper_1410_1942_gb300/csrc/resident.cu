@@ -33,7 +33,8 @@
 //
 // Several solves share one launch: the host gives each a set of CTAs and every CTA a list of
 // boxes ordered by one global order of the solves, so no two CTAs wait for each other's later
-// solves.  All waits are bounded (BAR_NS) and end the launch with the error flag set.
+// solves.  All waits are bounded (RES_WAIT_NS without progress anywhere in the launch) and end the
+// launch with the error flag set.
 #include "resident.h"
 
 #include <algorithm>
@@ -238,18 +239,30 @@ __device__ __forceinline__ double inv_of(double D) { return 1.0 / sqrt(D); }
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Bounded poll bookkeeping: false once the deadline has passed or another CTA has given up.
+// Bounded poll bookkeeping: false once the deadline has passed or another CTA has given up.  In a
+// launch of several solves the boxes waited for may belong to CTAs that are still in an earlier
+// solve of their lists: that is no fault however long it takes, so the deadline counts from the
+// launch's last sign of progress (which every solve gives each PROGRESS sweeps).  The iteration
+// caps bound the whole.
+constexpr unsigned PROGRESS = 16;
 struct Deadline {
-    unsigned spins = 0;
+    unsigned spins = 0, seen = 0;
     unsigned long long t0 = 0;
-    __device__ __forceinline__ bool more(int* error) {
+    __device__ __forceinline__ bool more(const ResArgs& a, unsigned long long limit) {
         if ((++spins & 63u) != 0) return true;
-        if (*(volatile int*)error) return false;
+        if (*(volatile int*)a.error) return false;
         const unsigned long long t = globaltimer();
-        if (!t0) t0 = t;
-        else if (t - t0 > BAR_NS) {
-            atomicExch(error, 1);
-            return false;
+        if (!t0) {
+            t0 = t;
+            seen = *(volatile unsigned*)a.progress;
+        } else if (t - t0 > limit) {
+            const unsigned now = *(volatile unsigned*)a.progress;
+            if (now == seen) {
+                atomicExch(a.error, 1);
+                return false;
+            }
+            seen = now;
+            t0 = t;
         }
         return true;
     }
@@ -456,6 +469,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
         for (;;) {
             ++tag;
             const unsigned par = tag & 1u;
+            if ((tag & (PROGRESS - 1)) == 0 && tk.rank == 0 && tid == 0) atomicAdd(a.progress, 1u);
             // w^ = M^-1 A u and the three sums
             V sg = (V)0, sd = (V)0, sr = (V)0;
             typename HW::W* const out = mine + par * half;
@@ -577,7 +591,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
 #pragma unroll
                         for (int q = 0; q < S::WORDS; ++q) all = all && S::is(wd[q], tag);
                         if (all) break;
-                        if (!dl.more(a.error)) { s_fail = 1; break; }
+                        if (!dl.more(a, sv.wait_ns)) { s_fail = 1; break; }
                     }
                     S::get(wd, t0, t1, t2);
                 }
@@ -707,7 +721,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
             if (late) {
                 Deadline dl;
                 while ((late = get_halo(late)) != 0)
-                    if (!dl.more(a.error)) { s_late = 1; break; }
+                    if (!dl.more(a, sv.wait_ns)) { s_late = 1; break; }
             }
 #pragma unroll
             for (int q = 0; q < HQ; ++q) {
@@ -971,7 +985,7 @@ struct Parts {
         solves = take(sizeof(ResSolve) * n);
         tasks = take(sizeof(ResTask) * b.tasks.size());
         cta = take(sizeof(int) * b.cta_task.size());
-        error = take(sizeof(int));
+        error = take(2 * sizeof(int));  // the error flag and the progress count
         sums = take(bytes_sums(n, dbl));
         outbox = take(bytes_out(b, dbl));
         bytes = at;
@@ -1035,6 +1049,7 @@ int res_plan_build(ResPlan* p, ResSolve* solves, int n, bool dbl, cudaStream_t s
     p->tasks = (ResTask*)(m + at.tasks);
     p->cta_task = (int*)(m + at.cta);
     p->error = (int*)(m + at.error);
+    p->progress = (unsigned*)(p->error + 1);
     p->sums = m + at.sums;
     p->outbox = m + at.outbox;
     p->words = p->sums;
@@ -1096,11 +1111,11 @@ int launch_res(const ResPlan& p, ResKind kind, const ResSolve* solves, int n, cu
                                      (int)(q == RES_FACES64 ? SMEM_MAX : smem_fix(depth)));
         cudaGetLastError();
     });
-    ResArgs a{p.solves, p.tasks, p.cta_task, p.sums, p.outbox, p.box_words, p.extra, p.error};
+    ResArgs a{p.solves, p.tasks, p.cta_task, p.sums, p.outbox, p.box_words, p.extra, p.error, p.progress};
     void* params[] = {&a};
     if (cudaMemcpyAsync(p.solves, solves, sizeof(ResSolve) * n, cudaMemcpyHostToDevice, st) !=
             cudaSuccess ||
-        cudaMemsetAsync(p.error, 0, sizeof(int), st) != cudaSuccess)
+        cudaMemsetAsync(p.error, 0, 2 * sizeof(int), st) != cudaSuccess)
         return -1;
     const cudaError_t e =
         coop_launch(kernel_of(kind, p.depth), dim3(p.ncta), dim3(RES_T), params, p.smem, st);

@@ -54,3 +54,35 @@ def test_an_unreachable_box_times_out_in_every_precision(prec, cut):
         _check(oracle.operator(c.F, apertures=aps), oracle.rhs(c.s, g.h, aps[3]), p, c.tol)
     else:
         _check(oracle.operator(c.F), oracle.rhs(c.s, g.h), p, c.tol)
+
+
+def test_a_box_that_waits_for_a_long_solve_before_it_is_no_timeout():
+    """One solve on nearly every SM with ten times the iterations its grid suggests, and small solves
+    dealt to its CTAs and the free ones: their first boxes wait for the long solve to end, with a
+    limit below that but above the distance of its signs of progress (16 sweeps, about 0.1 ms)."""
+    cases = [inputs.flat_case(160, 96, 80, seed=9, tol=1e-9)] + \
+            [inputs.flat_case(64, 48, 24 + i, seed=10 + i, tol=1e-9) for i in range(24)]
+    solvers, alone = [], []
+    for i, c in enumerate(cases):
+        g = c.grid
+        s = capi.Poisson(g.nx, g.ny, g.nz, g.h, inner_tol=1e-9 if i == 0 else 1e-4)
+        s.set_density(c.F)
+        assert "on chip" in s.describe(), s.describe()
+        p = np.zeros(g.shape)
+        assert s.solve(c.s, p, c.tol)[0] == capi.OK
+        s.test_wait_limit(1e-3)
+        solvers.append(s)
+        alone.append(p)
+    ps = [np.zeros(c.grid.shape) for c in cases]
+    rcs = []
+    for t in capi.batch_submit(solvers, [c.s for c in cases], ps, 1e-9):
+        while True:
+            rc, _ = capi.poll(t)
+            if rc != capi.PENDING:
+                break
+        rcs.append(rc)
+    for s in solvers:
+        s.close()
+    assert rcs == [capi.OK] * len(cases)
+    for p, q in zip(ps, alone):
+        assert np.linalg.norm(p - q) <= 2e-6 * np.linalg.norm(q)
