@@ -86,9 +86,10 @@ k_fine(const __grid_constant__ CUtensorMap mf0, const __grid_constant__ CUtensor
         fence_mbar_init();
         s_fail = 0;
     }
-    __syncthreads();
     pdl_entry();
-    if (a.sc && a.sc->done) return;
+    // (one answer for the whole block: a block of this grid whose wait runs out sets `done` meanwhile,
+    // and threads that left by themselves would be missing at the barriers below)
+    if (__syncthreads_or(a.sc && a.sc->done)) return;
     const Dims d = a.d;
     const int x0 = blockIdx.x * FW, y0 = blockIdx.y * FH;
     const int k0 = blockIdx.z * a.kc, k1 = min(d.nz, k0 + a.kc);
