@@ -362,6 +362,12 @@ int poisson_test_unreachable_box(poisson_t* h, int extra);
  * Errors: EINVAL (NULL, seconds not in (0, 1], not an on-chip handle). */
 int poisson_test_wait_limit(poisson_t* h, double seconds);
 
+/* The same kind of aid for the V-cycle's fine passes on TMA-staged planes: the blocks of one pass (1
+ * PCG phase A, 2 phase B, 3 restriction, 4 smoothing; 0 restores) never issue their last plane, so
+ * that their wait for it runs out (200 ms) and the call returns POISSON_ETIMEOUT.
+ * Errors: EINVAL (NULL, pass outside 0..4, a handle without these passes). */
+int poisson_test_withhold_plane(poisson_t* h, int pass);
+
 /* Testing aids for the allocation error paths (the failure is injected on the host; nothing
  * faults on the GPU).  poisson_test_fail_alloc(n): the n-th device or pinned-host allocation the
  * library makes from now on, in any thread, fails as if memory were exhausted, and the call that

@@ -35,7 +35,7 @@ EXPORTS = ["poisson_default_opts", "poisson_create", "poisson_destroy", "poisson
            "poisson_version", "poisson_test_unreachable_barrier", "poisson_hydrostatic_force",
            "poisson_required_bytes", "poisson_handle_bytes", "poisson_test_fail_alloc",
            "poisson_test_live_allocations", "poisson_test_unreachable_box",
-           "poisson_test_wait_limit"]
+           "poisson_test_wait_limit", "poisson_test_withhold_plane"]
 K_CG_A, K_CG_B, K_RESIDUAL, K_OTHER, K_PCG = 0, 1, 2, 3, 4
 K_NAMES = ["cg_phase_a", "cg_phase_b", "residual64", "other", "pcg_persistent"]
 
@@ -128,6 +128,8 @@ def load(path=None):
     lib.poisson_test_unreachable_box.restype = i
     lib.poisson_test_wait_limit.argtypes = [vp, d]
     lib.poisson_test_wait_limit.restype = i
+    lib.poisson_test_withhold_plane.argtypes = [vp, i]
+    lib.poisson_test_withhold_plane.restype = i
     lib.poisson_test_fail_alloc.argtypes = [i]
     lib.poisson_test_fail_alloc.restype = i
     lib.poisson_test_live_allocations.argtypes = [ctypes.POINTER(ctypes.c_longlong)]
@@ -275,6 +277,12 @@ class Poisson:
     def test_wait_limit(self, seconds):
         """Testing aid: how long the on-chip PCG's waits may see no progress (1 s by default)."""
         _check(load().poisson_test_wait_limit(self._h, float(seconds)), "poisson_test_wait_limit")
+
+    def test_withhold_plane(self, fine_pass):
+        """Testing aid: one fine pass of the V-cycle waits for a plane that never comes (1 phase A,
+        2 phase B, 3 restriction, 4 smoothing; 0 restores)."""
+        _check(load().poisson_test_withhold_plane(self._h, int(fine_pass)),
+               "poisson_test_withhold_plane")
 
     def device_bytes(self):
         """Device bytes the handle holds (poisson_handle_bytes)."""

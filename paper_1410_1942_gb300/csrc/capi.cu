@@ -1227,6 +1227,13 @@ extern "C" int poisson_test_wait_limit(poisson_t* H, double seconds) {
     return POISSON_OK;
 }
 
+extern "C" int poisson_test_withhold_plane(poisson_t* H, int pass) {
+    if (!H || pass < 0 || pass > 4 || !H->mg.fine) return POISSON_EINVAL;
+    drop_chunk_graph(H);  // it holds the launches' arguments
+    H->fine.withhold = pass;
+    return POISSON_OK;
+}
+
 extern "C" int poisson_solve(poisson_t* H, const double* rhs, double* p, double tol,
                              poisson_stats* stats) {
     if (!H || !rhs || !p || !(tol > 0.0)) return POISSON_EINVAL;
@@ -1262,6 +1269,9 @@ extern "C" int poisson_solve(poisson_t* H, const double* rhs, double* p, double 
             break;
     }
     if (status == POISSON_ECUDA) return status;
+    // A pass that gave up part way leaves its reduction's arrivals counted: the next reduction would
+    // take one of its blocks for the last before all partial sums are there.
+    if (status == POISSON_ETIMEOUT) CK(cudaMemsetAsync(H->sc, 0, sizeof(Scalars), H->st));
     CK(copy_user(p, H->x64, bytes, dp ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                        H->st));
     CK(cudaStreamSynchronize(H->st));

@@ -13,6 +13,8 @@ namespace pcg {
 struct FineMaps {
     bool on = false;
     bool bf16 = false;
+    int withhold = 0;  // testing aid: the pass (1 phase A, 2 phase B, 3 restriction, 4 smoothing) whose
+                       // blocks wait for a plane that never comes
     const float *z = nullptr, *pa = nullptr, *pb = nullptr, *x0 = nullptr, *r = nullptr, *x = nullptr;
     // halo boxes of z, both p buffers, x0 and rho/2; centre boxes of r and x
     CUtensorMap mz, mpa, mpb, mx0, meta, mr, mx;

@@ -86,3 +86,28 @@ def test_a_box_that_waits_for_a_long_solve_before_it_is_no_timeout():
     assert rcs == [capi.OK] * len(cases)
     for p, q in zip(ps, alone):
         assert np.linalg.norm(p - q) <= 2e-6 * np.linalg.norm(q)
+
+
+@pytest.mark.parametrize("fine_pass", [1, 2, 3, 4])
+def test_a_solve_after_a_fine_pass_timed_out_is_the_same_as_before(fine_pass):
+    """512 blocks a pass, more than are resident at once: the blocks of the first wave give up, those
+    of the second find the solve ended and leave without a word to the reduction.  The next solve on
+    the handle, of another source, gives bit for bit what it gave before."""
+    c = inputs.flat_case(1024, 512, 8, seed=11, tol=1e-9)
+    g = c.grid
+    other = inputs.flat_case(1024, 512, 8, seed=12, tol=1e-9).s * 1e-3
+    with capi.Poisson(g.nx, g.ny, g.nz, g.h, precond="mg") as s:
+        s.set_density(c.F)
+        ref = np.zeros(g.shape)
+        rc, st_ref = s.solve(other, ref, c.tol)
+        assert rc == capi.OK
+        s.test_withhold_plane(fine_pass)
+        p = np.zeros(g.shape)
+        rc, _ = s.solve(c.s, p, c.tol, allow=(capi.ETIMEOUT,))
+        assert rc == capi.ETIMEOUT and np.all(np.isfinite(p))
+        s.test_withhold_plane(0)
+        p = np.zeros(g.shape)
+        rc, st = s.solve(other, p, c.tol)
+        assert rc == capi.OK
+    assert st["outer_iters"] == st_ref["outer_iters"] and st["inner_iters"] == st_ref["inner_iters"]
+    assert st["rel_residual"] == st_ref["rel_residual"] and np.array_equal(p, ref)
