@@ -191,7 +191,8 @@ int poisson_apply(poisson_t* h, const double* x, double* y, int precision);
  * Jacobi M = D; SSOR M = (D - wE) D^{-1} (D - wE^T) / (w (2 - w)) in red-black order (red =
  * (i+j+k) even first, A = D - E - E^T); MG one V-cycle of the handle's hierarchy (only on a
  * POISSON_MG handle and at its own precision, else EINVAL; the FP32 cycle uses the handle's
- * inner FP32 vectors as scratch).  Errors: ENOTREADY, EINVAL, ECUDA. */
+ * inner FP32 vectors as scratch).  Errors: ENOTREADY, EINVAL, ECUDA, ETIMEOUT (a bounded wait of
+ * the FP32 cycle's fine passes ran out; z is unspecified). */
 int poisson_precond_apply(poisson_t* h, const double* r, double* z, int kind, int precision);
 
 /* Copy out the FP64 operator: low-side face coefficients bx, by, bz (bx[c] couples cell c with

@@ -1367,24 +1367,30 @@ extern "C" int poisson_precond_apply(poisson_t* H, const double* r, double* z, i
         if (precision == POISSON_FP64) {
             const CoefFaces64 c{H->bx, H->by, H->bz, H->diag, nullptr};
             return with_io(H, r, z, [&](const double* a, double* b) {
-                mg_apply<double, CoefFaces64>(&H->mg, d, kc, c, a, b, st);
+                mg_apply<double, CoefFaces64>(&H->mg, d, kc, c, a, b, nullptr, st);
             });
         }
         // FP32 V-cycle on narrowed copies (r32 and d32 are rebuilt by every solve)
-        return with_io(H, r, z, [&](const double* a, double* b) {
+        // (its fine passes on staged planes can time out: that is told by the scalars)
+        Scalars* const sc = H->mg.fine ? H->sc : nullptr;
+        const int rc = with_io(H, r, z, [&](const double* a, double* b) {
             launch_narrow_f32(d.n, a, H->r32, st);
             if (H->cut())
                 mg_apply<float, CoefFaces32>(&H->mg, d, kc,
                                              CoefFaces32{H->bx32, H->by32, H->bz32, H->diag32},
-                                             H->r32, H->d32, st);
+                                             H->r32, H->d32, sc, st);
             else if (precision == POISSON_FP32)
                 mg_apply<float, CoefEta<float>>(&H->mg, d, kc, CoefEta<float>{H->eta32}, H->r32,
-                                                H->d32, st);
+                                                H->d32, sc, st);
             else
                 mg_apply<float, CoefEta<__nv_bfloat16>>(
-                    &H->mg, d, kc, CoefEta<__nv_bfloat16>{H->eta16}, H->r32, H->d32, st);
+                    &H->mg, d, kc, CoefEta<__nv_bfloat16>{H->eta16}, H->r32, H->d32, sc, st);
             launch_widen_f32(d.n, H->d32, b, st);
         });
+        if (rc != POISSON_OK || !sc) return rc;
+        CK(cudaMemcpyAsync(&H->sc_host[0], sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        return H->sc_host[0].done == TIMEDOUT ? POISSON_ETIMEOUT : POISSON_OK;
     }
     const double om = H->opts.omega;
     if (kind == POISSON_RBSSOR) {

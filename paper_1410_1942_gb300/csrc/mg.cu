@@ -1322,12 +1322,13 @@ void mg_cg_b(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* p, V* 
 }
 
 template <typename V, typename Coef>
-void mg_apply(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z,
+void mg_apply(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z, Scalars* sc,
               cudaStream_t st) {
+    if (sc) cudaMemsetAsync(sc, 0, sizeof(Scalars), st);  // RUNNING
     launch_pdl(k_mg_first<V, Coef>, cols(d, kc), dim3(TX, TY), 0, st,
         d, coef, kc, r, (V*)m->x[0], (V)MG_OMEGA, nullptr, nullptr, 0.0, 0, 0);
     counted(1);
-    vcycle<V, Coef>(m, d, kc, coef, r, z, nullptr, nullptr, -1, st);
+    vcycle<V, Coef>(m, d, kc, coef, r, z, sc, nullptr, -1, st);
 }
 
 #define MG_INSTANTIATE(V, C)                                                                   \
@@ -1335,7 +1336,7 @@ void mg_apply(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V*
                                 double*, double, int, int, cudaStream_t);                      \
     template void mg_cg_b<V, C>(MgHier*, const Dims&, int, const C&, const V*, V*, V*, V*,     \
                                 Scalars*, double*, cudaStream_t);                              \
-    template void mg_apply<V, C>(MgHier*, const Dims&, int, const C&, const V*, V*,            \
+    template void mg_apply<V, C>(MgHier*, const Dims&, int, const C&, const V*, V*, Scalars*,  \
                                  cudaStream_t);
 
 MG_INSTANTIATE(double, CoefFaces64)

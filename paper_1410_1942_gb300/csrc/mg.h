@@ -63,8 +63,9 @@ void mg_init(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* 
 template <typename V, typename Coef>
 void mg_cg_b(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* p, V* x, V* r, V* z,
              Scalars* sc, double* part, cudaStream_t st);
+// z = V_0(r).  sc (or null): its `done` is TIMEDOUT afterwards if a wait of a pass ran out.
 template <typename V, typename Coef>
-void mg_apply(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z,
+void mg_apply(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z, Scalars* sc,
               cudaStream_t st);
 
 }  // namespace pcg

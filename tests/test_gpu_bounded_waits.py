@@ -111,3 +111,22 @@ def test_a_solve_after_a_fine_pass_timed_out_is_the_same_as_before(fine_pass):
         assert rc == capi.OK
     assert st["outer_iters"] == st_ref["outer_iters"] and st["inner_iters"] == st_ref["inner_iters"]
     assert st["rel_residual"] == st_ref["rel_residual"] and np.array_equal(p, ref)
+
+
+@pytest.mark.parametrize("fine_pass", [3, 4])
+def test_applying_the_v_cycle_reports_a_timed_out_pass(fine_pass):
+    """The V-cycle alone runs the restriction and the smoothing: a wait that runs out in one of them
+    is told, and the next application gives what it gave before."""
+    c = inputs.flat_case(64, 48, 32, seed=13)
+    with capi.Poisson(64, 48, 32, c.grid.h, precond="mg") as s:
+        s.set_density(c.F)
+        r = np.random.default_rng(1).standard_normal(c.grid.shape)
+        ref, z = np.empty_like(r), np.empty_like(r)
+        s.precond_apply(r, ref, "mg", "fp32")
+        s.test_withhold_plane(fine_pass)
+        with pytest.raises(capi.PoissonError) as e:
+            s.precond_apply(r, z, "mg", "fp32")
+        assert e.value.status == capi.ETIMEOUT
+        s.test_withhold_plane(0)
+        s.precond_apply(r, z, "mg", "fp32")
+        assert np.array_equal(z, ref)
