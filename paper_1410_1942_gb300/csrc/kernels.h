@@ -4,8 +4,30 @@
 #include "internal.cuh"
 
 #include <atomic>
+#include <mutex>
 
 namespace pcg {
+
+// Set-up that belongs to a device, such as a kernel's shared-memory attribute: run() calls f the
+// first time it is reached with each device current (with f done before anyone's run returns).
+class OncePerDevice {
+public:
+    template <typename F>
+    void run(F&& f) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+        const unsigned long long bit = 1ull << (dev & 63);
+        if (done_.load(std::memory_order_acquire) & bit) return;
+        std::lock_guard<std::mutex> lk(mu_);
+        if (done_.load(std::memory_order_relaxed) & bit) return;
+        f();
+        done_.fetch_or(bit, std::memory_order_release);
+    }
+
+private:
+    std::mutex mu_;
+    std::atomic<unsigned long long> done_{0};
+};
 
 // Launches kernel k with programmatic stream serialization: it may start launching while the
 // previous kernel of the stream drains (the kernel must begin with pdl_entry()).

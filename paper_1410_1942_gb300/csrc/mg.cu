@@ -7,7 +7,6 @@
 // the handle's reduction partials); the bottom levels and the coarsest run in one block.  Every
 // kernel of a PCG iteration returns at once when the solve has finished.
 #include <atomic>
-#include <mutex>
 
 #include "alloc.h"
 #include "poisson.h"
@@ -1136,8 +1135,8 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
     for (int q = 0; q < B.nb; ++q) T += B.d[q].n;
     const size_t smem = sizeof(V) * BOTTOM_ARRAYS * (size_t)T;
     if (smem <= BOTTOM_SMEM && B.d[B.nb - 1].n <= COARSE_T) {
-        static std::once_flag once;
-        std::call_once(once, [] {
+        static OncePerDevice once;
+        once.run([] {
             cudaFuncSetAttribute(k_mg_bottom_smem<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)BOTTOM_SMEM);
             cudaGetLastError();

@@ -21,7 +21,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "kernels.h"
 #include "march_dev.cuh"
@@ -397,8 +396,8 @@ dim3 fine_grid(const Dims& d, int kc) {
 template <int PASS>
 void launch(const FineMaps& m, const CUtensorMap& f0, const CUtensorMap& f1, const CUtensorMap& c0,
             const CUtensorMap& c1, FineArgs a, cudaStream_t st) {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static OncePerDevice once;
+    once.run([] {
         cudaFuncSetAttribute(k_fine<PASS, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              FGeo<PASS, float>::SMEM);
         cudaFuncSetAttribute(k_fine<PASS, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,

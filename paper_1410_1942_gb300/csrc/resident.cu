@@ -41,7 +41,6 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 
 #include "alloc.h"
 #include "coop.h"
@@ -1102,8 +1101,8 @@ int res_tags(ResPlan* p, ResSolve* solves, int n, cudaStream_t st) {
 }
 
 int launch_res(const ResPlan& p, ResKind kind, const ResSolve* solves, int n, cudaStream_t st) {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static OncePerDevice once;
+    once.run([] {
         for (int q = 0; q < 4; ++q)
             for (int depth : {2, 4, 8, 16})
                 cudaFuncSetAttribute(kernel_of((ResKind)q, depth),
