@@ -316,6 +316,9 @@ struct Executor {
             const int rc = res_plan_build(&rplan, h_res, nres, false, st);
             if (rc == -2) return POISSON_ENOMEM;
             if (rc != 0) return POISSON_EINVAL;
+            rplan.wait_ns = RES_WAIT_NS;
+            for (const Job* j : table)
+                if (j->h->res) rplan.wait_ns = std::min(rplan.wait_ns, j->h->rplan.wait_ns);
         }
         if (nmarch) {
             const int var = HB->march ? HB->plan.variant : 0;

@@ -359,7 +359,6 @@ ResSolve res_solve_of(const poisson_t* H) {
     s.r = dbl ? (const void*)H->r64 : (const void*)H->r32;
     s.x = dbl ? (void*)H->x64 : (void*)H->d32;
     s.ctas = H->res_host ? H->res_host->ctas : 0;
-    s.wait_ns = H->res_wait_ns;
     return s;
 }
 
@@ -1223,7 +1222,7 @@ extern "C" int poisson_test_unreachable_box(poisson_t* H, int extra) {
 
 extern "C" int poisson_test_wait_limit(poisson_t* H, double seconds) {
     if (!H || !H->res || !(seconds > 0.0) || seconds > 1.0) return POISSON_EINVAL;
-    H->res_wait_ns = (unsigned long long)(1e9 * seconds);
+    H->rplan.wait_ns = (unsigned long long)(1e9 * seconds);
     return POISSON_OK;
 }
 

@@ -83,7 +83,6 @@ struct poisson_s {
     bool res = false;
     pcg::ResPlan rplan{};
     pcg::ResSolve* res_host = nullptr;  // pinned staging of rplan.solves
-    unsigned long long res_wait_ns = pcg::RES_WAIT_NS;
     // a worker thread solves the handle beside others: no launch that fills the GPU
     bool no_coop = false;
     pcg::MarchPlan plan{};  // persistent work-list launch over this handle's grid

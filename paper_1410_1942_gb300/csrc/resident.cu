@@ -139,9 +139,7 @@ template <> struct Sum<float> {
     static __device__ __forceinline__ ff from_lane(ff v, int l) {
         return ff{__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
     }
-    static __device__ __forceinline__ bool is(const Word& w, unsigned tag) {
-        return (unsigned)(w.tag >> 32) == tag;
-    }
+    static __device__ __forceinline__ unsigned tag_of(const Word& w) { return (unsigned)(w.tag >> 32); }
     static __device__ __forceinline__ void get(const Word (&w)[WORDS], ff& g, ff& d, ff& r) {
         g = ff{__uint_as_float((unsigned)w[0].v), __uint_as_float((unsigned)(w[0].v >> 32))};
         d = ff{__uint_as_float((unsigned)w[0].tag), __uint_as_float((unsigned)w[1].v)};
@@ -164,9 +162,7 @@ template <> struct Sum<double> {
     static __device__ __forceinline__ double from_lane(double v, int l) {
         return __shfl_sync(0xffffffffu, v, l);
     }
-    static __device__ __forceinline__ bool is(const Word& w, unsigned tag) {
-        return (unsigned)w.tag == tag;
-    }
+    static __device__ __forceinline__ unsigned tag_of(const Word& w) { return (unsigned)w.tag; }
     static __device__ __forceinline__ void get(const Word (&w)[WORDS], double& g, double& d, double& r) {
         g = __longlong_as_double((long long)w[0].v);
         d = __longlong_as_double((long long)w[1].v);
@@ -238,31 +234,40 @@ __device__ __forceinline__ double inv_of(double D) { return 1.0 / sqrt(D); }
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Bounded poll bookkeeping: false once the deadline has passed or another CTA has given up.  In a
-// launch of several solves the boxes waited for may belong to CTAs that are still in an earlier
-// solve of their lists: that is no fault however long it takes, so the deadline counts from the
-// launch's last sign of progress (which every solve gives each PROGRESS sweeps).  The iteration
-// caps bound the whole.
-constexpr unsigned PROGRESS = 16;
+// Bounded poll bookkeeping: false once the deadline has passed or another CTA has given up.
 struct Deadline {
     unsigned spins = 0, seen = 0;
     unsigned long long t0 = 0;
-    __device__ __forceinline__ bool more(const ResArgs& a, unsigned long long limit) {
+    __device__ __forceinline__ bool more(int* error, unsigned long long limit) {
+        if ((++spins & 63u) != 0) return true;
+        if (*(volatile int*)error) return false;
+        const unsigned long long t = globaltimer();
+        if (!t0) t0 = t;
+        if (t - t0 <= limit) return true;
+        atomicExch(error, 1);
+        return false;
+    }
+    // The wait for a box's sums: the box may belong to a CTA that is still in an earlier solve of its
+    // list, which is no fault however long it takes.  It gives up only when no solve of the launch
+    // has begun a sweep during the second half of the limit, as the tags of their first boxes' sums
+    // tell.  The iteration caps bound the whole.
+    template <typename V>
+    __device__ __forceinline__ bool more_queued(const ResArgs& a, unsigned long long limit) {
         if ((++spins & 63u) != 0) return true;
         if (*(volatile int*)a.error) return false;
         const unsigned long long t = globaltimer();
-        if (!t0) {
-            t0 = t;
-            seen = *(volatile unsigned*)a.progress;
-        } else if (t - t0 > limit) {
-            const unsigned now = *(volatile unsigned*)a.progress;
-            if (now == seen) {
-                atomicExch(a.error, 1);
-                return false;
-            }
-            seen = now;
-            t0 = t;
+        if (!t0) t0 = t;
+        if (t - t0 <= limit / 2) return true;
+        unsigned now = 1;
+#pragma unroll 1
+        for (int q = 0; q < 2 * a.nsolves; ++q)  // both parities
+            now += Sum<V>::tag_of(ld_word((const Word*)a.sums + (size_t)RANKS * Sum<V>::STRIDE * q));
+        if (seen && now == seen) {
+            atomicExch(a.error, 1);
+            return false;
         }
+        seen = now;
+        t0 = t;
         return true;
     }
 };
@@ -468,7 +473,6 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
         for (;;) {
             ++tag;
             const unsigned par = tag & 1u;
-            if ((tag & (PROGRESS - 1)) == 0 && tk.rank == 0 && tid == 0) atomicAdd(a.progress, 1u);
             // w^ = M^-1 A u and the three sums
             V sg = (V)0, sd = (V)0, sr = (V)0;
             typename HW::W* const out = mine + par * half;
@@ -588,9 +592,9 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
 #pragma unroll
                         for (int q = 0; q < S::WORDS; ++q) wd[q] = ld_word(wv + q);
 #pragma unroll
-                        for (int q = 0; q < S::WORDS; ++q) all = all && S::is(wd[q], tag);
+                        for (int q = 0; q < S::WORDS; ++q) all = all && S::tag_of(wd[q]) == tag;
                         if (all) break;
-                        if (!dl.more(a, sv.wait_ns)) { s_fail = 1; break; }
+                        if (!dl.more_queued<V>(a, a.wait_ns)) { s_fail = 1; break; }
                     }
                     S::get(wd, t0, t1, t2);
                 }
@@ -720,7 +724,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
             if (late) {
                 Deadline dl;
                 while ((late = get_halo(late)) != 0)
-                    if (!dl.more(a, sv.wait_ns)) { s_late = 1; break; }
+                    if (!dl.more(a.error, a.wait_ns)) { s_late = 1; break; }
             }
 #pragma unroll
             for (int q = 0; q < HQ; ++q) {
@@ -984,7 +988,7 @@ struct Parts {
         solves = take(sizeof(ResSolve) * n);
         tasks = take(sizeof(ResTask) * b.tasks.size());
         cta = take(sizeof(int) * b.cta_task.size());
-        error = take(2 * sizeof(int));  // the error flag and the progress count
+        error = take(sizeof(int));
         sums = take(bytes_sums(n, dbl));
         outbox = take(bytes_out(b, dbl));
         bytes = at;
@@ -1048,7 +1052,6 @@ int res_plan_build(ResPlan* p, ResSolve* solves, int n, bool dbl, cudaStream_t s
     p->tasks = (ResTask*)(m + at.tasks);
     p->cta_task = (int*)(m + at.cta);
     p->error = (int*)(m + at.error);
-    p->progress = (unsigned*)(p->error + 1);
     p->sums = m + at.sums;
     p->outbox = m + at.outbox;
     p->words = p->sums;
@@ -1110,11 +1113,12 @@ int launch_res(const ResPlan& p, ResKind kind, const ResSolve* solves, int n, cu
                                      (int)(q == RES_FACES64 ? SMEM_MAX : smem_fix(depth)));
         cudaGetLastError();
     });
-    ResArgs a{p.solves, p.tasks, p.cta_task, p.sums, p.outbox, p.box_words, p.extra, p.error, p.progress};
+    ResArgs a{p.solves, p.tasks, p.cta_task, p.sums, p.outbox, p.box_words, p.extra, p.error, p.nsolves,
+              p.wait_ns};
     void* params[] = {&a};
     if (cudaMemcpyAsync(p.solves, solves, sizeof(ResSolve) * n, cudaMemcpyHostToDevice, st) !=
             cudaSuccess ||
-        cudaMemsetAsync(p.error, 0, 2 * sizeof(int), st) != cudaSuccess)
+        cudaMemsetAsync(p.error, 0, sizeof(int), st) != cudaSuccess)
         return -1;
     const cudaError_t e =
         coop_launch(kernel_of(kind, p.depth), dim3(p.ncta), dim3(RES_T), params, p.smem, st);

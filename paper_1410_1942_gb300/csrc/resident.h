@@ -28,7 +28,6 @@ struct ResSolve {
     int active;    // 0: skipped; its scalars come back CONVERGED with 0 iterations
     double tol2;   // stop when r.r <= tol2 (b.b for RES_FACES64, else r0.r0)
     int max_iter;
-    unsigned long long wait_ns;  // a wait without progress in the launch gives up after this
     unsigned tag0;  // the solve's sweeps carry the tags tag0 + 1, tag0 + 2, ... (res_tags)
 };
 
@@ -50,10 +49,11 @@ struct ResArgs {
     int box_words;
     int extra;            // > 0: wait for one box more than there are (a testing aid)
     int* error;           // set to 1 once a wait has run out
-    unsigned* progress;   // counted up by every solve each few sweeps
+    int nsolves;
+    unsigned long long wait_ns;  // a wait without progress in the launch gives up after this
 };
 
-constexpr unsigned long long RES_WAIT_NS = 1000ull * 1000ull * 1000ull;  // ResSolve::wait_ns: 1 s
+constexpr unsigned long long RES_WAIT_NS = 1000ull * 1000ull * 1000ull;  // 1 s
 constexpr int RES_MAX_CTAS = 159;  // boxes of one solve (one more reduction word for the test aid)
 
 struct ResPlan {
@@ -62,6 +62,7 @@ struct ResPlan {
     size_t smem = 0;  // dynamic shared memory of the launch
     bool dbl = false;
     int extra = 0;
+    unsigned long long wait_ns = RES_WAIT_NS;
     unsigned next_tag = 0;
     // one device allocation, carved into:
     void* mem = nullptr;
@@ -70,7 +71,6 @@ struct ResPlan {
     ResTask* tasks = nullptr;
     int* cta_task = nullptr;
     int* error = nullptr;
-    unsigned* progress = nullptr;
     void* words = nullptr;  // the tagged words: sums, then outbox
     size_t words_bytes = 0;
     void* sums = nullptr;

@@ -59,7 +59,7 @@ def test_an_unreachable_box_times_out_in_every_precision(prec, cut):
 def test_a_box_that_waits_for_a_long_solve_before_it_is_no_timeout():
     """One solve on nearly every SM with ten times the iterations its grid suggests, and small solves
     dealt to its CTAs and the free ones: their first boxes wait for the long solve to end, with a
-    limit below that but above the distance of its signs of progress (16 sweeps, about 0.1 ms)."""
+    limit below that but above the time of its sweeps (0.5 ms holds about 60)."""
     cases = [inputs.flat_case(160, 96, 80, seed=9, tol=1e-9)] + \
             [inputs.flat_case(64, 48, 24 + i, seed=10 + i, tol=1e-9) for i in range(24)]
     solvers, alone = [], []
