@@ -211,6 +211,10 @@ __device__ __forceinline__ ff ff_div(ff a, ff b) {
     return ff{h, __fsub_rn(q2, __fsub_rn(h, q))};
 }
 
+__device__ __forceinline__ bool ff_le(ff a, ff b) {
+    return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo);
+}
+
 template <typename Coef> __device__ __forceinline__ Coef coef_of(const ResSolve& s);
 template <> __device__ __forceinline__ CoefEta<float> coef_of(const ResSolve& s) {
     return CoefEta<float>{(const float*)s.c[0]};
@@ -298,6 +302,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
     __shared__ T red[RES_W][3];
     __shared__ T tot[RANKS / 32][3];
     __shared__ double s_dec[2];
+    __shared__ ff s_stop;  // FP32: stop when r.r is at most this
     __shared__ int s_state, s_iter;
     // A wait that ran out: for a sum, written before the decision's barrier and read after it; for a
     // halo word, written after that barrier and read after the sweep's last one.  One flag for
@@ -462,7 +467,6 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
         // scalars: in FP32 every thread holds them (float-float); in FP64 warp 0 decides
         T gam = S::of((V)0), den = S::of((V)0);
         V al = (V)0, be = (V)0;
-        float stop_f = 0.f;
         bool first = true;
         int iter = 0, state = RUNNING;
         double rr_out = 0.0, rz_out = 0.0;
@@ -608,6 +612,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
             if (late) late = get_halo(late);
             if constexpr (!DBL) {
                 ff g = tot[0][0], dl = tot[0][1], r = tot[0][2];
+                const ff stop_at = s_stop;  // (set by the first decision)
                 for (int q = 1; 32 * q < nwait; ++q) {
                     g = ff_add(g, tot[q][0]);
                     dl = ff_add(dl, tot[q][1]);
@@ -620,9 +625,11 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
                     state = BREAKDOWN;
                 } else if (first) {
                     first = false;
-                    stop_f = (float)tol2 * r.hi;
+                    const float th = (float)tol2;
+                    const ff stop = ff_mul(ff{th, (float)(tol2 - (double)th)}, r);
+                    if (tid == 0) s_stop = stop;
                     gam = g;
-                    if (r.hi <= stop_f) state = CONVERGED;
+                    if (ff_le(r, stop)) state = CONVERGED;
                     else if (!(dl.hi > 0.f)) state = BREAKDOWN;
                     else {
                         den = dl;
@@ -631,7 +638,7 @@ __global__ void __launch_bounds__(RES_T, 1) k_res(ResArgs a) {
                     }
                 } else {
                     ++iter;
-                    if (r.hi <= stop_f) state = CONVERGED;
+                    if (ff_le(r, stop_at)) state = CONVERGED;
                     else if (iter >= max_iter) state = CAPPED;
                     else {
                         // beta = gamma'/gamma, alpha = gamma' / (delta' - beta^2 den)
