@@ -364,9 +364,9 @@ int poisson_test_unreachable_box(poisson_t* h, int extra);
 int poisson_test_wait_limit(poisson_t* h, double seconds);
 
 /* The same kind of aid for the V-cycle's fine passes on TMA-staged planes: the blocks of one pass (1
- * PCG phase A, 2 phase B, 3 restriction, 4 smoothing; 0 restores) never issue their last plane, so
- * that their wait for it runs out (200 ms) and the call returns POISSON_ETIMEOUT.
- * Errors: EINVAL (NULL, pass outside 0..4, a handle without these passes). */
+ * PCG phase A, 2 phase B, 3 restriction, 4 smoothing; 0 restores) load planes that are a row short, so
+ * that their waits for whole planes run out (200 ms) and the call returns POISSON_ETIMEOUT.
+ * Errors: EINVAL (NULL, pass outside 0..4, a handle without these passes), ECUDA. */
 int poisson_test_withhold_plane(poisson_t* h, int pass);
 
 /* Testing aids for the allocation error paths (the failure is injected on the host; nothing

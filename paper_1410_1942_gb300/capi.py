@@ -279,7 +279,7 @@ class Poisson:
         _check(load().poisson_test_wait_limit(self._h, float(seconds)), "poisson_test_wait_limit")
 
     def test_withhold_plane(self, fine_pass):
-        """Testing aid: one fine pass of the V-cycle waits for a plane that never comes (1 phase A,
+        """Testing aid: one fine pass of the V-cycle waits for planes that stay a row short (1 phase A,
         2 phase B, 3 restriction, 4 smoothing; 0 restores)."""
         _check(load().poisson_test_withhold_plane(self._h, int(fine_pass)),
                "poisson_test_withhold_plane")

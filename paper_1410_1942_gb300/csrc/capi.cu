@@ -1229,8 +1229,7 @@ extern "C" int poisson_test_wait_limit(poisson_t* H, double seconds) {
 extern "C" int poisson_test_withhold_plane(poisson_t* H, int pass) {
     if (!H || pass < 0 || pass > 4 || !H->mg.fine) return POISSON_EINVAL;
     drop_chunk_graph(H);  // it holds the launches' arguments
-    H->fine.withhold = pass;
-    return POISSON_OK;
+    return fine_maps_withhold(&H->fine, H->d, pass) ? POISSON_OK : POISSON_ECUDA;
 }
 
 extern "C" int poisson_solve(poisson_t* H, const double* rhs, double* p, double tol,

@@ -57,7 +57,6 @@ struct FineArgs {
     int kc;         // planes per block (even)
     int fz, sz;     // restriction, smoothing: the aggregates' factor and shift along z
     int mode;       // smoothing: as k_mg_smooth
-    int withhold;   // testing aid: the last plane of a block is never issued
     float alpha, omega;
     const float* e;      // smoothing: the coarse correction
     const float* cdiag;  // restriction
@@ -100,7 +99,6 @@ k_fine(const __grid_constant__ CUtensorMap mf0, const __grid_constant__ CUtensor
             // planes k0 - 1 .. k1; the centre boxes of the planes computed
             const int L = k1 - k0;
             for (int q = 0; q < L + 2; ++q) {
-                if (a.withhold && q == L + 1) break;
                 const int st = q % FNS, k = k0 - 1 + q;
                 if (q >= FNS && !mbar_wait_or(&empty[st], ((q / FNS) - 1) & 1, &s_fail)) {
                     s_fail = 1;
@@ -394,8 +392,9 @@ dim3 fine_grid(const Dims& d, int kc) {
 }
 
 template <int PASS>
-void launch(const FineMaps& m, const CUtensorMap& f0, const CUtensorMap& f1, const CUtensorMap& c0,
+void launch(const FineMaps& m, const CUtensorMap& field, const CUtensorMap& f1, const CUtensorMap& c0,
             const CUtensorMap& c1, FineArgs a, cudaStream_t st) {
+    const CUtensorMap& f0 = m.withhold == PASS + 1 ? m.mshort : field;
     static OncePerDevice once;
     once.run([] {
         cudaFuncSetAttribute(k_fine<PASS, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -405,7 +404,6 @@ void launch(const FineMaps& m, const CUtensorMap& f0, const CUtensorMap& f1, con
         cudaGetLastError();
     });
     a.kc = fine_kc(a.d);
-    a.withhold = m.withhold == PASS + 1;
     const dim3 grid = fine_grid(a.d, a.kc);
     if (m.bf16)
         launch_pdl(k_fine<PASS, __nv_bfloat16>, grid, dim3(FTHREADS), FGeo<PASS, __nv_bfloat16>::SMEM,
@@ -437,6 +435,12 @@ bool fine_maps_build(FineMaps* m, const Dims& d, const void* eta, bool bf16, con
             march_encode_box(&m->mr, r, false, d, FW, FH) &&
             march_encode_box(&m->mx, x, false, d, FW, FH);
     return m->on;
+}
+
+bool fine_maps_withhold(FineMaps* m, const Dims& d, int pass) {
+    if (pass && !march_encode_box(&m->mshort, m->z, false, d, FW + 8, FH + 1)) return false;
+    m->withhold = pass;
+    return true;
 }
 
 void launch_fine_a(const FineMaps& m, const Dims& d, bool in_a, float* p_out, Scalars* sc,

@@ -13,11 +13,10 @@ namespace pcg {
 struct FineMaps {
     bool on = false;
     bool bf16 = false;
-    int withhold = 0;  // testing aid: the pass (1 phase A, 2 phase B, 3 restriction, 4 smoothing) whose
-                       // blocks wait for a plane that never comes
+    int withhold = 0;  // testing aid (fine_maps_withhold): the pass whose planes stay incomplete
     const float *z = nullptr, *pa = nullptr, *pb = nullptr, *x0 = nullptr, *r = nullptr, *x = nullptr;
     // halo boxes of z, both p buffers, x0 and rho/2; centre boxes of r and x
-    CUtensorMap mz, mpa, mpb, mx0, meta, mr, mx;
+    CUtensorMap mz, mpa, mpb, mx0, meta, mr, mx, mshort;
 };
 
 // Whether the passes serve a grid: rows of whole 32 bytes, no wrap, no stored faces, aggregates of
@@ -27,6 +26,10 @@ bool fine_maps_fit(const Dims& d);
 bool fine_maps_build(FineMaps* m, const Dims& d, const void* eta, bool bf16, const float* z,
                      const float* pa, const float* pb, const float* x0, const float* r,
                      const float* x);
+
+// Testing aid: the boxes that one pass (1 phase A, 2 phase B, 3 restriction, 4 smoothing; 0: none)
+// loads of its field are a row short, so that its waits for the full planes run out.
+bool fine_maps_withhold(FineMaps* m, const Dims& d, int pass);
 
 // The passes (launched with programmatic stream serialization): phase A, phase B, the finest
 // restriction and the finest post-smoothing, as k_cg_a, k_mg_cg_b, k_mg_restrict and k_mg_smooth.
