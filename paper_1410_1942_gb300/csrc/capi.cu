@@ -789,16 +789,19 @@ extern "C" int poisson_set_density(poisson_t* H, const double* F, double rho_air
         CK(copy_user(H->b64, F, bytes, cudaMemcpyHostToDevice, H->st));
         Fd = H->b64;
     }
-    // the density check's flag lives in the reduction partials (free between solves)
+    // the density checks' flags live in the reduction partials (free between solves)
     unsigned* bad = reinterpret_cast<unsigned*>(H->partials);
-    CK(cudaMemsetAsync(bad, 0, sizeof(unsigned), H->st));
+    CK(cudaMemsetAsync(bad, 0, 2 * sizeof(unsigned), H->st));
     H->ready = false;
     launch_setup(H->d, Fd, rho_air, rho_water, H->bx, H->by, H->bz, H->diag, H->dinv, H->top64,
-                 H->rinv2, H->eta32, H->eta16, H->apertures(), bad, H->st);
-    unsigned bad_host = 0;
-    CK(cudaMemcpyAsync(&bad_host, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, H->st));
+                 H->rinv2, H->eta32, H->eta16, H->apertures(), MG_PLAIN_RHO, bad, H->st);
+    unsigned bad_host[2] = {0, 0};
+    CK(cudaMemcpyAsync(bad_host, bad, sizeof bad_host, cudaMemcpyDeviceToHost, H->st));
     CK(cudaStreamSynchronize(H->st));
-    if (bad_host) return POISSON_EINVAL;  // left not ready: solves give ENOTREADY
+    if (bad_host[0]) return POISSON_EINVAL;  // left not ready: solves give ENOTREADY
+    const bool plain = bad_host[1] || std::min(rho_air, rho_water) < MG_PLAIN_RHO;
+    if (plain != H->mg.plain) drop_chunk_graph(H);  // other kernels
+    H->mg.plain = plain;
     if (H->pitched()) {
         if (H->peta32) launch_pitch_rows(H->d, H->pitch, H->eta32, H->peta32, H->st);
         if (H->peta16) launch_pitch_rows(H->d, H->pitch, H->eta16, H->peta16, H->st);

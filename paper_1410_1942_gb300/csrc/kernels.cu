@@ -84,7 +84,8 @@ __device__ __forceinline__ int phase_of(double F) {
 // Dirichlet side/bottom wall the cell touches, x-, x+, y-, y+, z-), summed in that order;
 // top[i + nx j] = 2/rho_c of the top layer; rinv2[c] = 2/rho_c (only with Dirichlet walls).
 // bad: set to 1 when some cell's density is not a positive finite number (F non-finite, or so
-// far outside [0, 1] that rho <= 0): the operator is then not SPD.
+// far outside [0, 1] that rho <= 0): the operator is then not SPD.  bad[1]: when some cell's density
+// is below `tiny`, cells of pure phase aside.
 //
 // Bound by the FP64 pipe (two operations a clock and SM) wherever it divides: three divisions a
 // face pass and two a diagonal pass took 301 and 127 us on 256x128x128, against 30 us for the
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(256) k_setup(Dims d, FastDiv by_nx, FastDiv by
                                                double* __restrict__ dinv, double* __restrict__ top,
                                                double* __restrict__ rinv2, float* __restrict__ eta32,
                                                __nv_bfloat16* __restrict__ eta16, Apertures ap,
-                                               unsigned* __restrict__ bad) {
+                                               double tiny, unsigned* __restrict__ bad) {
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (tid >= d.n) return;
     const int c = (int)tid;
@@ -132,7 +133,8 @@ __global__ void __launch_bounds__(256) k_setup(Dims d, FastDiv by_nx, FastDiv by
         return;
     }
     const double rc = rho_of(Fc, ra, rw);
-    if (!(rc > 0.0) || !isfinite(rc)) *bad = 1u;
+    if (!(rc > 0.0) || !isfinite(rc)) bad[0] = 1u;
+    if (rc < tiny) bad[1] = 1u;
     const bool act = !ap.vol || ap.vol[c] > 0.0;
     // the face to a neighbour: 0 if there is none; with cut cells scaled by its open fraction, and
     // closed next to a cell with no fluid
@@ -1041,11 +1043,11 @@ static inline unsigned blocks1d(long long n) { return (unsigned)((n + 255) / 256
 
 void launch_setup(const Dims& d, const double* F, double ra, double rw, double* bx, double* by,
                   double* bz, double* diag, double* dinv, double* top, double* rinv2,
-                  float* eta32, __nv_bfloat16* eta16, const Apertures& ap, unsigned* bad,
-                  cudaStream_t st) {
+                  float* eta32, __nv_bfloat16* eta16, const Apertures& ap, double tiny,
+                  unsigned* bad, cudaStream_t st) {
     k_setup<<<blocks1d(d.n), 256, 0, st>>>(d, FastDiv(d.nx), FastDiv(d.ny), F, ra, rw,
                                            phases_of(ra, rw), bx, by, bz, diag, dinv, top, rinv2,
-                                           eta32, eta16, ap, bad);
+                                           eta32, eta16, ap, tiny, bad);
     counted(1);
 }
 

@@ -1065,7 +1065,11 @@ __global__ void __launch_bounds__(TX * TY) k_mg_cg_b(Dims d, Coef coef, int kc,
 }
 
 // Whether the fine passes run on TMA-staged planes (the handle's maps are for this residual).
-inline bool fine_of(const MgHier& m, const float* r) { return m.fine && m.fine->r == r; }
+inline bool fine_of(const MgHier& m, const float* r) {
+    return m.fine && m.fine->r == r && !m.plain;
+}
+// ... or with 2 x 2 cells per thread (both divide by div_refined).
+inline bool quads_of(const MgHier& m, const Dims& d) { return quad_tiles_fit(d) && !m.plain; }
 
 // z = V_0(r) given x[0] = w D^-1 r: restrictions down, the coarsest sweeps, prolongation +
 // post-smoothing up; the fine smoothing writes z (and reduces r.z when mode >= 0).
@@ -1148,7 +1152,7 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
     for (int l = b - 1; l >= 1; --l) {
         const int* f = m->f[l];
         if constexpr (std::is_same<V, float>::value) {
-            if (quad_tiles_fit(m->d[l])) {
+            if (quads_of(*m, m->d[l])) {
                 launch_pdl(k_mg_smooth_fq, quad_grid(m->d[l], quad_kc(m->d[l], QB_FACES)),
                            dim3(TX, TY), 0, st, m->d[l], LevelCoef<float>::of(*m, l),
                            quad_kc(m->d[l], QB_FACES), (const V*)m->r[l], (const V*)m->x[l],
@@ -1167,7 +1171,7 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
         if (fine_of(*m, r))
             launch_fine_smooth(*m->fine, d, m->d[1], f[2] - 1, (const float*)m->y[1], al, om, z, sc,
                                part, mode, st);
-        else if (quad_tiles_fit(d))
+        else if (quads_of(*m, d))
             launch_pdl(k_mg_smooth_q<EtaOf<Coef>>, quad_grid(d, quad_kc(d, QB_SMOOTH)), dim3(TX, TY),
                        0, st, d, coef, quad_kc(d, QB_SMOOTH), r, (const V*)m->x[0], (const V*)m->y[1], m->d[1], f[2] - 1,
                 al, om, z, sc, part, mode);
@@ -1179,7 +1183,7 @@ void vcycle(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* r, V* z
             launch_pdl(k_mg_smooth_eta<EtaOf<Coef>>, cols(d, kc), dim3(TX, TY), 0, st,
                 d, coef, kc, r, (const V*)m->x[0], (const V*)m->y[1], m->d[1], f[0] - 1,
                 f[1] - 1, f[2] - 1, al, om, z, sc, part, mode);
-    } else if (std::is_same<Coef, CoefFaces32>::value && quad_tiles_fit(d)) {
+    } else if (std::is_same<Coef, CoefFaces32>::value && quads_of(*m, d)) {
         launch_pdl(k_mg_smooth_fq, quad_grid(d, quad_kc(d, QB_FACES)), dim3(TX, TY), 0, st, d,
                    faces32_of(coef), quad_kc(d, QB_FACES), (const float*)r,
                    (const float*)m->x[0], (const float*)m->y[1], m->d[1], f[2] - 1, (float)al,
@@ -1297,7 +1301,7 @@ void mg_cg_b(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* p, V* 
         if (fine_of(*m, r))
             launch_fine_b(*m->fine, d, p == m->fine->pa, x, r, (float*)m->x[0], (float)MG_OMEGA, sc,
                           part, st);
-        else if (quad_tiles_fit(d))
+        else if (quads_of(*m, d))
             launch_pdl(k_mg_cg_b_q<EtaOf<Coef>>, quad_grid(d, quad_kc(d, QB_CG_B)), dim3(TX, TY), 0,
                        st, d, coef, quad_kc(d, QB_CG_B), p, x, r, (V*)m->x[0], (V)MG_OMEGA, sc, part);
         else if (plane_tiles_fit(d))
@@ -1308,7 +1312,7 @@ void mg_cg_b(MgHier* m, const Dims& d, int kc, const Coef& coef, const V* p, V* 
             launch_pdl(k_mg_cg_b_eta<EtaOf<Coef>>, cols(d, kc), dim3(TX, TY), 0, st, d, coef, kc, p, x, r,
                                                                 (V*)m->x[0], (V)MG_OMEGA, sc,
                                                                 part);
-    } else if (std::is_same<Coef, CoefFaces32>::value && quad_tiles_fit(d)) {
+    } else if (std::is_same<Coef, CoefFaces32>::value && quads_of(*m, d)) {
         launch_pdl(k_mg_cg_b_fq, quad_grid(d, quad_kc(d, QB_FACES)), dim3(TX, TY), 0, st, d,
                    faces32_of(coef), quad_kc(d, QB_FACES), (const float*)p, (float*)x, (float*)r,
                    (float*)m->x[0], (float)MG_OMEGA, sc, part);

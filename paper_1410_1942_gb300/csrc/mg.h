@@ -26,6 +26,8 @@ namespace pcg {
 constexpr int MG_MAX_LEVELS = 32;
 constexpr double MG_OMEGA = 0.9;   // Jacobi smoother damping
 constexpr double MG_ALPHA = 1.5;   // coarse-correction scaling
+// (a diagonal is at most 12/rho, a coarse one at most the sum of its fewer than 2^31 cells')
+constexpr double MG_PLAIN_RHO = 0x1p-90;
 constexpr int MG_COARSE_MAX = 512;
 constexpr int MG_COARSE_SWEEPS = 16;
 
@@ -33,6 +35,9 @@ struct FineMaps;
 
 struct MgHier {
     const FineMaps* fine = nullptr;  // the fine passes on TMA-staged planes (mg_tma.h), or null
+    // Some density is below MG_PLAIN_RHO: a level's diagonal may pass 2^126, where div_refined fails, and
+    // the updates take the passes that divide.
+    bool plain = false;
     int nlev = 0;     // levels, the fine one included (>= 2 once planned)
     bool dbl = false;  // level arrays in FP64 (FP64 handles) or FP32
     Dims d[MG_MAX_LEVELS] = {};

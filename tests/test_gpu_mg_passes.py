@@ -85,3 +85,22 @@ def test_bottom_levels_match_the_oracle(shape, walls, prec):
         got = np.empty_like(r)
         s.precond_apply(r, got, kind="mg", precision=prec)
     assert np.linalg.norm(got - want) <= VCYCLE_TOL[prec] * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("periodic", [False, True])
+def test_densities_whose_diagonal_has_a_flushed_reciprocal(periodic):
+    """Diagonals of 1.3 * 2^126, whose FP32 reciprocal is below the normal numbers: the damped-Jacobi
+    updates divide by them all the same.  p scales with the density."""
+    shape = (1, 2, 64)
+    rho = 6 / (2.0 ** 126 * 1.3)
+    F = np.zeros(shape)
+    b = np.random.default_rng(1).standard_normal(shape) * 1e10
+    out = []
+    for r in (1.0, rho):
+        with capi.Poisson(64, 2, 1, 0.1, precond="mg", periodic_x=periodic, max_iters=300) as s:
+            s.set_density(F, r, r)
+            p = np.zeros(shape)
+            rc, _ = s.solve(b, p, 1e-9, allow=(capi.OK, capi.ENOTCONV))
+            assert rc == capi.OK, r
+            out.append(p / r)
+    assert np.linalg.norm(out[1] - out[0]) <= 1e-6 * np.linalg.norm(out[0])
