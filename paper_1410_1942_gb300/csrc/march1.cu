@@ -250,14 +250,19 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                         wzl[y][x] = (sg.k0 > 0 || (d.walls & 16)) ? rcp_approx(ec[y][x] + em[y][x]) : 0.f;
             }
             float ag = 0.f, ad = 0.f, ar = 0.f;
-            // the thread's arrays and its cell of the plane: read from the record again after every
-            // store, which may alias it, they made an iteration 30.2 us on 256x128x128 (29.9 now),
-            // 119.7 on 512x256x128 with BF16 densities (116.4) and 22.8 on 250x125x90 (21.7)
-            const int rp = MODE != ROWS_PLAIN ? s_sol[l].nxp : d.nx;  // u, s^ and w^'s row
+            // the thread's arrays and its cell of the plane, kept over the planes: read from the record
+            // again after every store, which may alias it, they made an iteration 30.2 us on
+            // 256x128x128 (29.9 now), 119.7 on 512x256x128 with BF16 densities (116.4) and 22.8 on
+            // 250x125x90 (21.7).  The FP32 kernel of the 64x16 tile (96 registers a thread) has no
+            // room for them: 36.6 us on 256x128x128 with them kept, 35.3 read again
+            constexpr bool KEEP = TYT < 8 || sizeof(E) == 2;
+            const LocalSolve1& Lr = s_sol[l];
+            const int rp = MODE != ROWS_PLAIN ? Lr.nxp : d.nx;  // u, s^ and w^'s row
             size_t cell = (size_t)i0 + (size_t)(PER ? d.nx : rp) * (j0 + (size_t)d.ny * sg.k0);
-            float *const gx = s_sol[l].x, *const gp = s_sol[l].p, *const gu = s_sol[l].u[out],
-                  *const gs = s_sol[l].s[out], *const gw = s_sol[l].w[out];
-            for (int k = sg.k0; k < sg.k1; ++k, cell += (size_t)(PER ? d.nx : rp) * d.ny) {
+            float *const kx = Lr.x, *const kp = Lr.p, *const ku = Lr.u[out], *const ks = Lr.s[out],
+                  *const kw = Lr.w[out];
+            auto row_now = [&] { return KEEP ? rp : MODE != ROWS_PLAIN ? s_sol[l].nxp : d.nx; };
+            for (int k = sg.k0; k < sg.k1; ++k, cell += KEEP ? (size_t)(PER ? d.nx : rp) * d.ny : 0) {
                 const int qc = p0 + 1 + (k - sg.k0), qn = qc + 1;
                 ok = acquire();  // plane k+1
                 if (ok && work) {
@@ -314,21 +319,23 @@ __global__ void __launch_bounds__(32 * (TYT + 1), WsMinBlocks<TYT>::value) k_cg1
                                     ad += in ? qv[y][x] * uc[y][x] : 0.f;
                                     ar += du * du;
                                 }
-                                const size_t c = cell + (size_t)(PER ? d.nx : rp) * y;
-                                if (xs) st_row<CX>(gx + c, xn);
-                                st_row<CX>(gp + c, pn);
-                                const size_t row = PER ? (size_t)rp * (j0 + y + (size_t)d.ny * k) : 0;
+                                const size_t c = KEEP ? cell + (size_t)(PER ? d.nx : rp) * y
+                                                      : (size_t)i0 + (size_t)(PER ? d.nx : row_now()) *
+                                                                         (j0 + y + (size_t)d.ny * k);
+                                if (xs) st_row<CX>((KEEP ? kx : s_sol[l].x) + c, xn);
+                                st_row<CX>((KEEP ? kp : s_sol[l].p) + c, pn);
+                                const size_t row = PER ? (size_t)row_now() * (j0 + y + (size_t)d.ny * k) : 0;
                                 const size_t cp = PER ? row + i0 + PAD_V : c;
-                                st_row<CX>(gu + cp, uc[y]);
-                                st_row<CX>(gs + cp, sn);
-                                st_row<CX>(gw + cp, wn);
+                                st_row<CX>((KEEP ? ku : s_sol[l].u[out]) + cp, uc[y]);
+                                st_row<CX>((KEEP ? ks : s_sol[l].s[out]) + cp, sn);
+                                st_row<CX>((KEEP ? kw : s_sol[l].w[out]) + cp, wn);
                                 if (PER && (i0 < PAD_V || i0 >= d.nx - PAD_V)) {
                                     // the ghost copy at the other end of the padded row
                                     const long long cg = (long long)row + i0 + PAD_V +
                                                          (i0 < PAD_V ? d.nx : -d.nx);
-                                    st_row<CX>(gu + cg, uc[y]);
-                                    st_row<CX>(gs + cg, sn);
-                                    st_row<CX>(gw + cg, wn);
+                                    st_row<CX>((KEEP ? ku : s_sol[l].u[out]) + cg, uc[y]);
+                                    st_row<CX>((KEEP ? ks : s_sol[l].s[out]) + cg, sn);
+                                    st_row<CX>((KEEP ? kw : s_sol[l].w[out]) + cg, wn);
                                 }
                             }
                         }
