@@ -369,6 +369,10 @@ int poisson_test_wait_limit(poisson_t* h, double seconds);
  * Errors: EINVAL (NULL, pass outside 0..4, a handle without these passes), ECUDA. */
 int poisson_test_withhold_plane(poisson_t* h, int pass);
 
+/* The blocks that the handle's reductions have counted so far; 0 between calls, or the next reduction
+ * would end before its last block.  Errors: EINVAL (NULL), ECUDA. */
+int poisson_test_counted_arrivals(poisson_t* h, unsigned* count);
+
 /* Testing aids for the allocation error paths (the failure is injected on the host; nothing
  * faults on the GPU).  poisson_test_fail_alloc(n): the n-th device or pinned-host allocation the
  * library makes from now on, in any thread, fails as if memory were exhausted, and the call that

@@ -35,7 +35,8 @@ EXPORTS = ["poisson_default_opts", "poisson_create", "poisson_destroy", "poisson
            "poisson_version", "poisson_test_unreachable_barrier", "poisson_hydrostatic_force",
            "poisson_required_bytes", "poisson_handle_bytes", "poisson_test_fail_alloc",
            "poisson_test_live_allocations", "poisson_test_unreachable_box",
-           "poisson_test_wait_limit", "poisson_test_withhold_plane"]
+           "poisson_test_wait_limit", "poisson_test_withhold_plane",
+           "poisson_test_counted_arrivals"]
 K_CG_A, K_CG_B, K_RESIDUAL, K_OTHER, K_PCG = 0, 1, 2, 3, 4
 K_NAMES = ["cg_phase_a", "cg_phase_b", "residual64", "other", "pcg_persistent"]
 
@@ -130,6 +131,8 @@ def load(path=None):
     lib.poisson_test_wait_limit.restype = i
     lib.poisson_test_withhold_plane.argtypes = [vp, i]
     lib.poisson_test_withhold_plane.restype = i
+    lib.poisson_test_counted_arrivals.argtypes = [vp, ctypes.POINTER(ctypes.c_uint)]
+    lib.poisson_test_counted_arrivals.restype = i
     lib.poisson_test_fail_alloc.argtypes = [i]
     lib.poisson_test_fail_alloc.restype = i
     lib.poisson_test_live_allocations.argtypes = [ctypes.POINTER(ctypes.c_longlong)]
@@ -283,6 +286,13 @@ class Poisson:
         2 phase B, 3 restriction, 4 smoothing; 0 restores)."""
         _check(load().poisson_test_withhold_plane(self._h, int(fine_pass)),
                "poisson_test_withhold_plane")
+
+    def test_counted_arrivals(self):
+        """Testing aid: blocks counted by an unfinished reduction (0 between calls)."""
+        n = ctypes.c_uint(0)
+        _check(load().poisson_test_counted_arrivals(self._h, ctypes.byref(n)),
+               "poisson_test_counted_arrivals")
+        return int(n.value)
 
     def device_bytes(self):
         """Device bytes the handle holds (poisson_handle_bytes)."""

@@ -1235,6 +1235,13 @@ extern "C" int poisson_test_withhold_plane(poisson_t* H, int pass) {
     return fine_maps_withhold(&H->fine, H->d, pass) ? POISSON_OK : POISSON_ECUDA;
 }
 
+extern "C" int poisson_test_counted_arrivals(poisson_t* H, unsigned* count) {
+    if (!H || !count) return POISSON_EINVAL;
+    CK(cudaStreamSynchronize(H->st));
+    CK(cudaMemcpy(count, &H->sc->ticket, sizeof *count, cudaMemcpyDeviceToHost));
+    return POISSON_OK;
+}
+
 extern "C" int poisson_solve(poisson_t* H, const double* rhs, double* p, double tol,
                              poisson_stats* stats) {
     if (!H || !rhs || !p || !(tol > 0.0)) return POISSON_EINVAL;

@@ -90,7 +90,7 @@ def test_a_box_that_waits_for_a_long_solve_before_it_is_no_timeout():
 
 @pytest.mark.parametrize("fine_pass", [1, 2, 3, 4])
 def test_a_solve_after_a_fine_pass_timed_out_is_the_same_as_before(fine_pass):
-    """512 blocks a pass, more than are resident at once: the blocks of the first wave give up, those
+    """512 tiles a pass, more blocks than are resident at once: the blocks of the first wave give up, those
     of the second find the solve ended and leave without a word to the reduction.  The next solve on
     the handle, of another source, gives bit for bit what it gave before."""
     c = inputs.flat_case(1024, 512, 8, seed=11, tol=1e-9)
@@ -105,6 +105,7 @@ def test_a_solve_after_a_fine_pass_timed_out_is_the_same_as_before(fine_pass):
         p = np.zeros(g.shape)
         rc, _ = s.solve(c.s, p, c.tol, allow=(capi.ETIMEOUT,))
         assert rc == capi.ETIMEOUT and np.all(np.isfinite(p))
+        assert s.test_counted_arrivals() == 0
         s.test_withhold_plane(0)
         p = np.zeros(g.shape)
         rc, st = s.solve(other, p, c.tol)
