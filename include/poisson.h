@@ -93,13 +93,14 @@ typedef struct {
     double inner_tol;  /* FP32 inner solve: relative residual reduction per refinement step
                           (default 1e-4; ignored by POISSON_FP64)                                  */
     int tile;          /* inner-solve kernels.  0 = Jacobi-PCG on chip when the grid fits the
-                          registers and shared memory of the GPU (about 1.2 million cells in
-                          FP32, half of that in FP64); else, FP32, the TMA plane-marching kernels,
-                          variant and z-chunk autotuned per shape (rows whose nx is not a multiple
-                          of 8 on the one-sweep ones, at a padded pitch; with periodic_x or red-black
-                          SSOR those rows take the column kernels); -1 = column kernels (plain loads); 10000000 F + 1000000 P +
-                          100000 S + 10000 WS + 1000 CX + 100 CY + T = persistent marching
-                          kernel with T rows of 32 threads, each owning CX x CY cells (tile
+                          registers and shared memory of the GPU (every ship-tank shape of up to
+                          0.8 million cells in FP32 and 0.5 million in FP64, some up to 1.2 and
+                          0.6 million); else, FP32, the TMA plane-marching kernels, variant and
+                          z-chunk autotuned per shape (rows whose nx is not a multiple of 8 on the
+                          one-sweep ones, at a padded pitch; with periodic_x or red-black SSOR
+                          those rows take the column kernels); -1 = column kernels (plain loads);
+                          10000000 F + 1000000 P + 100000 S + 10000 WS + 1000 CX + 100 CY + T =
+                          persistent marching kernel with T rows of 32 threads, each owning CX x CY cells (tile
                           32 CX x CY T), a TMA producer warp when WS = 1 and an S-stage plane
                           ring (S omitted = 4).  F = 0, two sweeps per CG iteration: 1108, 2204,
                           2208, 12204, 12208, 302204, 302208, 312208, 602204, 612208; F = 1, one
@@ -119,8 +120,8 @@ typedef struct {
                           face is corrected with 1/rho_c over the half cell.                    */
     int periodic_x;    /* 1: x periodic (the cells i = 0 and i = nx-1 of a row are neighbours
                           through the face x = 0 = Lx, as in the paper's strut run); no x walls
-                          then (EINVAL with POISSON_WALL_XM/XP), red-black SSOR needs an even nx,
-                          and the inner solve runs on the column kernels.  Face arrays of
+                          then (EINVAL with POISSON_WALL_XM/XP); red-black SSOR needs an even nx
+                          and takes the column kernels.  Face arrays of
                           poisson_divergence / poisson_project keep nx+1 x-faces; faces 0 and nx
                           are the same face (poisson_project writes both).  Default 0.         */
 } poisson_opts;
@@ -204,8 +205,8 @@ int poisson_get_operator(poisson_t* h, double* bx, double* by, double* bz, doubl
  * Many independent solves of uneven size driven together.  Every FP64 refinement step of the
  * batch is one batched residual kernel, one batched CG start and ONE cooperative persistent
  * PCG launch over all unfinished solves that stream their grids, and one over those held on
- * chip (captured in CUDA graphs, rebuilt when the batch changes).  Solves submitted while a batch runs join it at its next refinement step
- * (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or periodic x that
+ * chip (captured in CUDA graphs, rebuilt when the batch changes).  Solves submitted while a batch
+ * runs join it at its next refinement step (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or periodic x that
  * neither fits on chip nor has nx % 8 == 0 are solved with poisson_solve on worker threads;
  * POISSON_RBSSOR and periodic handles that stream one by one when polled.
  * poisson_batch_submit enqueues n solves (handles[i] with its density already set, rhs[i],
@@ -349,8 +350,9 @@ int poisson_residual_noalloc(int nx, int ny, int nz, double h, const double* F, 
  * leaves, and poisson_solve returns POISSON_ETIMEOUT with p holding the iterate reached.  The
  * CUDA context stays usable; extra = 0 restores normal launches.  It exists so that tests can
  * exercise the bounded-wait failure path without faulting or hanging the GPU.
- * Errors: EINVAL (NULL, extra < 0 or > 1024, or a handle whose inner solve does not use a
- * persistent launch: POISSON_FP64, RBSSOR, MG, cut cells, nx % 8 != 0, tile = -1). */
+ * Errors: EINVAL (NULL, extra < 0 or > 1024, or a handle whose inner solve is not a persistent
+ * FP32 launch: POISSON_FP64, MG, cut cells, tile = -1, and RBSSOR or periodic x on grids that take
+ * the column kernels). */
 int poisson_test_unreachable_barrier(poisson_t* h, int extra);
 
 /* The same for a handle whose PCG runs on chip, of any precision and with cut cells: with extra = 1

@@ -510,8 +510,7 @@ bool poolable(const poisson_t* H) { return !H->march && !H->rb; }
 // handle's device current and runs poisson_solve on a non-blocking stream of its own (ordered
 // after the caller's work on the handle's stream by an event recorded at submit; the handle's
 // stream is restored afterwards), then publishes the result under g_mu.  Own streams let the
-// jobs overlap on the GPU even when their handles run on the legacy default stream, and let the
-// CG loop replay its chunk graph (a legacy stream cannot be captured).
+// jobs overlap on the GPU even when their handles run on the legacy default stream.
 constexpr int N_WORKERS = 8;
 
 struct Pool {

@@ -1,7 +1,9 @@
 // resident.cu -- Jacobi-preconditioned CG with the whole state of a solve on chip.
 //
-// A grid of up to about 1.2 million cells (FP32; half that in FP64) fits the registers and shared
-// memory of the GPU's SMs.  One CTA of 512 threads per SM holds a box of the grid for a whole
+// A grid whose boxes, one an SM, fit the registers and shared memory is held there: on 152 SMs every
+// ship-tank shape (width and depth 0.35 to 0.75 of the length) of up to 0.8 million cells in FP32 and
+// 0.5 million in FP64, half of them at 1.0 and 0.55 million, and only shapes that are nearly whole
+// boxes up to 1.2 and 0.6 million.  One CTA of 512 threads per SM holds a box of the grid for a whole
 // inner solve: a thread owns one x-y column of the box (up to 16 planes in FP32, 8 in FP64) with
 // x, p, s^ and w^ in registers; u with a one-cell halo, the three low faces and the diagonal lie
 // in shared memory.  The recurrences are the Chronopoulos-Gear form of march1.cu (one reduction
@@ -28,8 +30,13 @@
 // the words, decision) and 0.3 us per plane of a box (shared-memory loads: eleven a cell); FP64,
 // the FP64 pipe (fifteen operations a cell) and the exchange's FP64 additions.  Measured against the
 // streamed and column kernels it replaces, us per iteration: FP32 64x48x32 3.5 against 8.3,
-// 128x64x64 4.3 against 11.3, 160x96x80 7.3 (169 Gcell-iterations/s) against 15.0, odd 123x55x43
-// 4.4 against 34.6; FP64 32^3 7.1 against 18.6, 128x64x64 22.2 against 62.
+// 128x64x64 4.3 against 11.4, 160x96x80 6.7 (182 Gcell-iterations/s) against 15.1, odd 123x55x43
+// 4.4 against 34.7; FP64 32^3 7.1 against 18.3, 128x64x64 22.4 against 63 (a solve's time over its
+// iterations; inside the launches alone 2.98, 3.94, 6.60, 3.85, 7.2 and 21.8).
+//
+// The scalars of the FP32 recurrences (alpha, beta, the denominator, the stopping test) are
+// float-float, about 2^-44, formed by every thread.  Formed in FP64 by one lane they gave bit for bit
+// the same pressure on 120 of 120 random grids, at 0.8 to 2 us more an iteration.
 //
 // Several solves share one launch: the host gives each a set of CTAs and every CTA a list of
 // boxes ordered by one global order of the solves, so no two CTAs wait for each other's later
