@@ -206,9 +206,11 @@ int poisson_get_operator(poisson_t* h, double* bx, double* by, double* bz, doubl
  * batch is one batched residual kernel, one batched CG start and ONE cooperative persistent
  * PCG launch over all unfinished solves that stream their grids, and one over those held on
  * chip (captured in CUDA graphs, rebuilt when the batch changes).  Solves submitted while a batch
- * runs join it at its next refinement step (continuous batching).  Handles with POISSON_FP64, POISSON_MG, cut cells or periodic x that
- * neither fits on chip nor has nx % 8 == 0 are solved with poisson_solve on worker threads;
- * POISSON_RBSSOR and periodic handles that stream one by one when polled.
+ * runs join it at its next refinement step (continuous batching).  Handles with POISSON_FP64,
+ * POISSON_MG, cut cells or periodic x that neither fits on chip nor has nx % 8 == 0 are solved with
+ * poisson_solve on worker threads (a Jacobi handle among them on the column kernels even where
+ * poisson_solve by itself runs it on chip); POISSON_RBSSOR and periodic handles that stream one by
+ * one when polled.
  * poisson_batch_submit enqueues n solves (handles[i] with its density already set, rhs[i],
  * p[i] in/out as in poisson_solve, tol[i]) and returns a ticket per solve.  The arrays must stay
  * valid, and the handles must not be used or destroyed, until poisson_poll reports the ticket.

@@ -157,7 +157,8 @@ __device__ __forceinline__ void quad_apply(const Quad& u, const Quad& e, const Q
 // (Markstein's refinement).  The correction's own error is about 2^-22 of an ulp, so this is the
 // rounded quotient except for those that close to the middle of two numbers (one in 80 million random
 // pairs); a fraction of the instructions of an IEEE division, which cost a solve on 1024x512x256
-// 1.2 % and one with cut cells on 192x96x96 1.6 %.  Above 2^126 the reciprocal is flushed to zero: MgHier::plain keeps such diagonals away.
+// 1.2 % and one with cut cells on 192x96x96 1.6 %.  Above 2^126 the reciprocal is flushed to zero:
+// MgHier::plain keeps such diagonals away.
 __device__ __forceinline__ float div_refined(float n, float d) {
     const float y = rcp_approx(d);
     const float q = n * y;
