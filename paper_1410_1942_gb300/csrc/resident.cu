@@ -129,7 +129,7 @@ template <> struct Halo<double> {
 template <typename V> struct Sum;
 template <> struct Sum<float> {
     using T = ff;
-    static constexpr int WORDS = 2, STRIDE = 2;
+    static constexpr int WORDS = 2, STRIDE = 2, TAG_AT = 3;  // (tag_of's 32 bits of a word)
     static __device__ __forceinline__ ff of(float v) { return ff{v, 0.f}; }
     static __device__ __forceinline__ ff add(ff a, ff b) { return ff_add(a, b); }
     static __device__ __forceinline__ ff shfl(ff v, int m) {
@@ -155,7 +155,7 @@ template <> struct Sum<float> {
 };
 template <> struct Sum<double> {
     using T = double;
-    static constexpr int WORDS = 3, STRIDE = 4;
+    static constexpr int WORDS = 3, STRIDE = 4, TAG_AT = 2;
     static __device__ __forceinline__ double of(double v) { return v; }
     static __device__ __forceinline__ double add(double a, double b) { return a + b; }
     static __device__ __forceinline__ double shfl(double v, int m) {
@@ -250,11 +250,11 @@ struct Deadline {
     unsigned spins = 0, seen = 0;
     unsigned long long t0 = 0;
     __device__ __forceinline__ bool more(int* error, unsigned long long limit) {
-        if ((++spins & 63u) != 0) return true;
+        if (__builtin_expect((++spins & 63u) != 0, 1)) return true;
         if (*(volatile int*)error) return false;
         const unsigned long long t = globaltimer();
         if (!t0) t0 = t;
-        if (t - t0 <= limit) return true;
+        if (__builtin_expect(t - t0 <= limit, 1)) return true;
         atomicExch(error, 1);
         return false;
     }
@@ -264,15 +264,16 @@ struct Deadline {
     // tell.  The iteration caps bound the whole.
     template <typename V>
     __device__ __forceinline__ bool more_queued(const ResArgs& a, unsigned long long limit) {
-        if ((++spins & 63u) != 0) return true;
+        if (__builtin_expect((++spins & 63u) != 0, 1)) return true;
         if (*(volatile int*)a.error) return false;
         const unsigned long long t = globaltimer();
         if (!t0) t0 = t;
-        if (t - t0 <= limit / 2) return true;
+        if (__builtin_expect(t - t0 <= limit / 2, 1)) return true;
         unsigned now = 1;
 #pragma unroll 1
         for (int q = 0; q < 2 * a.nsolves; ++q)  // both parities
-            now += Sum<V>::tag_of(ld_word((const Word*)a.sums + (size_t)RANKS * Sum<V>::STRIDE * q));
+            now += ((const volatile unsigned*)a.sums)[4 * (size_t)RANKS * Sum<V>::STRIDE * q +
+                                                      Sum<V>::TAG_AT];
         if (seen && now == seen) {
             atomicExch(a.error, 1);
             return false;
