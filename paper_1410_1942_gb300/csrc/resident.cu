@@ -32,7 +32,7 @@
 // streamed and column kernels it replaces, us per iteration: FP32 64x48x32 3.5 against 8.3,
 // 128x64x64 4.3 against 11.4, 160x96x80 6.7 (182 Gcell-iterations/s) against 15.1, odd 123x55x43
 // 4.4 against 34.7; FP64 32^3 7.1 against 18.3, 128x64x64 22.4 against 63 (a solve's time over its
-// iterations; inside the launches alone 2.98, 3.94, 6.60, 3.85, 7.2 and 21.8).
+// iterations; inside the launches alone 2.96, 3.93, 6.61, 3.84, 7.2 and 21.8).
 //
 // The scalars of the FP32 recurrences (alpha, beta, the denominator, the stopping test) are
 // float-float, about 2^-44, formed by every thread.  Formed in FP64 by one lane they gave bit for bit
